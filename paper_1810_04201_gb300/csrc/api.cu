@@ -47,7 +47,7 @@ size_t gauge_dir_bytes(const wd_ctx *c, Prec p) { return round_up(link_dir_bytes
 template <int P, int RECON>
 static void gauge_pack(const double *canon, void *dst, const Geom &g, size_t dir, cudaStream_t st) {
     dim3 grid((g.V + 127) / 128, 4);
-    k_gauge_pack<P, RECON><<<grid, 128, 0, st>>>(reinterpret_cast<const double2 *>(canon), dst, g.V, g.Vs, dir);
+    k_gauge_pack<P, RECON><<<grid, 128, 0, st>>>(reinterpret_cast<const double2 *>(canon), dst, g.V, g.Vs, dir, g.links_fx);
 }
 
 wd_status gauge_get(wd_ctx *c, Prec p, const void **out) {
@@ -91,6 +91,24 @@ wd_status check_recon8(wd_ctx *c, const char *who) {
     if (!(nmin >= 1e-6f))
         return fail(c, WD_ERR_ARG, std::string(who) + ": recon 8 needs |U01|^2 + |U02|^2 >= 1e-6 on every link "
                                    "(smallest: " + std::to_string(nmin) + "); use recon 12 or 18");
+    return WD_OK;
+}
+
+// Geom::links_fx for the canonical copy: every link unitary
+static wd_status check_unitary(wd_ctx *c) {
+    void *w;
+    wd_status s = ws_get(c, "gauge_check", sizeof(unsigned), &w);
+    if (s != WD_OK) return s;
+    WD_CUDA(c, cudaMemsetAsync(w, 0, sizeof(unsigned), c->stream));
+    const size_t nl = (size_t)4 * c->g.V;
+    k_gauge_not_unitary<<<(int)std::min<size_t>((nl + 255) / 256, 4096), 256, 0, c->stream>>>(
+        reinterpret_cast<const double2 *>(c->gauge_canon), nl, static_cast<unsigned *>(w));
+    WD_CUDA(c, cudaGetLastError());
+    c->launches += 1;
+    unsigned bad = 0;
+    WD_CUDA(c, cudaMemcpyAsync(&bad, w, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
+    WD_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->g.links_fx = bad ? 0 : 1;
     return WD_OK;
 }
 
@@ -241,6 +259,7 @@ wd_status wd_create(wd_ctx **out, const int dims[4], int antiperiodic_t, void *s
     c->g.eo_parity = -1;
     c->g.dbg = nullptr;
     c->g.split_t = 0;
+    c->g.links_fx = 0;
     c->stream = (cudaStream_t)stream;
     if (cudaGetDevice(&c->device) != cudaSuccess) {
         delete c;
@@ -298,9 +317,11 @@ wd_status wd_set_gauge(wd_ctx *c, const double *U, int on_device, int recon) {
         wd_status s = check_recon8(c, "wd_set_gauge");
         if (s != WD_OK) return s;
     }
+    wd_status s = check_unitary(c);
+    if (s != WD_OK) return s;
     c->has_gauge = true;
     const void *d;
-    wd_status s = gauge_get(c, F64, &d);
+    s = gauge_get(c, F64, &d);
     if (s != WD_OK) return s;
     if (!on_device) WD_CUDA(c, cudaStreamSynchronize(c->stream));
     return WD_OK;

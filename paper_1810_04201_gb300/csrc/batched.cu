@@ -173,14 +173,7 @@ __device__ void for_tiles_half(const BatchArgs &a, W &&want, F &&body) {
 template <int RECON, bool DAG>
 __device__ __forceinline__ void hop64_half(const LatDesc &L, const void *in, int s, int hh, bool on,
                                            C<double> (&own)[6]) {
-    C<double> acc[9];
-    if (on) hopping_half<F64, RECON, DAG, false, false>(L.g, in, L.g64, L.gdir64, s, hh, acc);
-    else
-#pragma unroll
-        for (int k = 0; k < 9; ++k) acc[k] = C<double>{0.0, 0.0};
-    exchange_halves(acc);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) own[k] = acc[k];
+    hopping_own<F64, RECON, DAG, false, false>(L.g, in, L.g64, L.gdir64, s, hh, on, own);
 }
 
 // Five blocks of 128 threads per SM (96 registers): the inner FP32 phases, which wait on

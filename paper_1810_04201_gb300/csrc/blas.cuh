@@ -146,8 +146,9 @@ template <int P> __global__ void k_zero(VecArgs v) {
 
 // One link, canonical complex128 u[9] -> the layout of precision P and recon R,
 // at index idx of arrays with stride Vs starting at `base` (one direction).
+// fx (FP64, recon 18 and 12): as fixed-point limbs.
 template <int P, int RECON>
-__device__ __forceinline__ void pack_link(const double2 *u, char *base, int Vs, int idx) {
+__device__ __forceinline__ void pack_link(const double2 *u, char *base, int Vs, int idx, bool fx) {
     if constexpr (RECON == 8) {
         // entries 1, 2, 3 and the phases of entries 0 and 6
         const double th0 = atan2(u[0].y, u[0].x), th6 = atan2(u[6].y, u[6].x);
@@ -177,8 +178,16 @@ __device__ __forceinline__ void pack_link(const double2 *u, char *base, int Vs, 
     }
     constexpr int n = RECON == 12 ? 6 : 9;
     if (P == F64) {
-        double2 *d = reinterpret_cast<double2 *>(base) + idx;
-        for (int e = 0; e < n; ++e) d[(size_t)e * Vs] = u[e];
+        if (fx) {
+            int4 *d = reinterpret_cast<int4 *>(base) + idx;
+            for (int e = 0; e < n; ++e) {
+                const int2 re = fx_link(u[e].x), im = fx_link(u[e].y);
+                d[(size_t)e * Vs] = make_int4(re.x, re.y, im.x, im.y);
+            }
+        } else {
+            double2 *d = reinterpret_cast<double2 *>(base) + idx;
+            for (int e = 0; e < n; ++e) d[(size_t)e * Vs] = u[e];
+        }
     } else if (P == DF32) {
         float4 *d = reinterpret_cast<float4 *>(base) + idx;
         for (int e = 0; e < n; ++e) {
@@ -212,10 +221,39 @@ __device__ __forceinline__ void pack_link(const double2 *u, char *base, int Vs, 
 
 // gauge: canonical (4 x V x 9 complex128, device) -> field of precision P, recon R
 template <int P, int RECON> __global__ void k_gauge_pack(const double2 *canon, void *dst, int V, int Vs,
-                                                         size_t dir_bytes) {
+                                                         size_t dir_bytes, int fx) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (s >= V) return;
-    pack_link<P, RECON>(canon + ((size_t)mu * V + s) * 9, reinterpret_cast<char *>(dst) + (size_t)mu * dir_bytes, Vs, s);
+    pack_link<P, RECON>(canon + ((size_t)mu * V + s) * 9, reinterpret_cast<char *>(dst) + (size_t)mu * dir_bytes, Vs, s,
+                        fx != 0);
+}
+
+// *bad = 1 when the rows of some link are not orthonormal to 2^-11 (NaN included): the
+// fixed-point FP64 arithmetic needs unitary links (fixed64.cuh)
+template <int DUMMY = 0> __global__ void k_gauge_not_unitary(const double2 *canon, size_t nlinks, unsigned *bad) {
+    for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += (size_t)gridDim.x * blockDim.x) {
+        float2 u[9];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const double2 t = canon[l * 9 + e];
+            u[e] = make_float2((float)t.x, (float)t.y);
+        }
+        bool ok = true;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = i; j < 3; ++j) {
+                float re = i == j ? -1.f : 0.f, im = 0.f;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float2 a = u[3 * i + k], b = u[3 * j + k];
+                    re += a.x * b.x + a.y * b.y;
+                    im += a.x * b.y - a.y * b.x;
+                }
+                ok &= fabsf(re) < 0x1p-11f && fabsf(im) < 0x1p-11f;
+            }
+        if (!ok) *bad = 1u;
+    }
 }
 
 // smallest n = |u01|^2 + |u02|^2 over all links (the recon-8 denominator), as the
@@ -242,7 +280,7 @@ template <int P, int RECON> __global__ void k_gauge_pack_eo(const double2 *canon
     const int t = rem / g.L[2];
     const int par = (x + y + z + t) & 1;
     char *base = reinterpret_cast<char *>(dst) + (size_t)(4 * par + mu) * dir_bytes;
-    pack_link<P, RECON>(canon + ((size_t)mu * g.V + n) * 9, base, Vhs, n >> 1);
+    pack_link<P, RECON>(canon + ((size_t)mu * g.V + n) * 9, base, Vhs, n >> 1, g.links_fx != 0);
 }
 
 __device__ __forceinline__ int site_parity(const Geom &g, int n) {

@@ -127,7 +127,7 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const void *in, const cha
         C<R> p[12], h[6], w[6], u[9];
         SpinorIO<P>::template load<NC>(in, g.Vs, sf, p);
         project<MU, SF>(p, h);
-        LinkIO<P, RECON>::load(gdir, g.Vs, s, u);
+        load_link<P, RECON>(g, gdir, g.Vs, s, u);
         su3_mult<false>(u, h, w, MU == 3 && g.antiperiodic && c == L - 1);
         if (MU == 3 && g.split_t && c == L - 1) zero6(w);  // the neighbour lives on the next sub-lattice
         accumulate<MU, SF>(acc, w);
@@ -137,7 +137,7 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const void *in, const cha
         C<R> p[12], h[6], w[6], u[9];
         SpinorIO<P>::template load<NC>(in, g.Vs, sb, p);
         project<MU, -SF>(p, h);
-        LinkIO<P, RECON>::load(gdir, g.Vs, sb, u);
+        load_link<P, RECON>(g, gdir, g.Vs, sb, u);
         su3_mult<true>(u, h, w, MU == 3 && g.antiperiodic && c == 0);
         if (MU == 3 && g.split_t && c == 0) zero6(w);  // the neighbour lives on the previous sub-lattice
         accumulate<MU, -SF>(acc, w);
@@ -348,7 +348,7 @@ __device__ __forceinline__ void hop_dir_eo(const Geom &g, const void *in, const 
             C<R> p[12], h[6], w[6], u[9];
             SpinorIO<P>::template load<NC>(in, g.Vs, nf >> 1, p);
             project<MU, SF>(p, h);
-            LinkIO<P, RECON>::load(gp, g.Vs, k, u);
+            load_link<P, RECON>(g, gp, g.Vs, k, u);
             su3_mult<false>(u, h, w, MU == 3 && g.antiperiodic && c == L - 1);
             accumulate<MU, SF>(acc, w);
         }
@@ -357,7 +357,7 @@ __device__ __forceinline__ void hop_dir_eo(const Geom &g, const void *in, const 
             C<R> p[12], h[6], w[6], u[9];
             SpinorIO<P>::template load<NC>(in, g.Vs, nb >> 1, p);
             project<MU, -SF>(p, h);
-            LinkIO<P, RECON>::load(gq, g.Vs, nb >> 1, u);
+            load_link<P, RECON>(g, gq, g.Vs, nb >> 1, u);
             su3_mult<true>(u, h, w, MU == 3 && g.antiperiodic && c == 0);
             accumulate<MU, -SF>(acc, w);
         }
@@ -381,9 +381,9 @@ __device__ __forceinline__ void hopping_eo(const Geom &g, const void *in, const 
 }
 
 // ---------------------------------------------------------------- two lanes per site
-// FP64 is bound by the FP64 units, which belong to the four schedulers of an SM:
-// a scheduler without warps leaves its unit idle, as in the partial last wave of a
-// launch.  So FP64 sites run on two lanes of a warp, lane l and l ^ 16, and twice
+// FP64 and DF32 are bound by arithmetic on units that belong to the four schedulers of
+// an SM: a scheduler without warps leaves its units idle, as in the partial last wave of
+// a launch.  So their sites run on two lanes of a warp, lane l and l ^ 16, and twice
 // as many warps share the work.  DF32 (bound by instruction issue) does the same:
 // half the work per lane needs 128 instead of 255 registers, so twice the warps
 // hide the latencies.  Lane half hh computes spin component hh of every
@@ -463,10 +463,11 @@ __device__ __forceinline__ void su3_mult1(const C<R> (&u)[9], const C<R> (&h)[3]
 // LO = 3 for mu = 0, 1 and 6 for mu = 2, 3 selects the accumulator block of spin ps.
 
 template <int P, int RECON, bool DAG, int LO, bool NC, class R>
-__device__ __forceinline__ void half_pair(int mu, const void *in, int Vs, int nf, const char *gf, int kf, bool flip_f,
+__device__ __forceinline__ void half_pair(const Geom &g, int mu, const void *in, int nf, const char *gf, int kf, bool flip_f,
                                           int nb, const char *gb, int kb, bool flip_b, int hh, C<R> (&acc)[9],
                                           bool zero_f = false, bool zero_b = false) {
     constexpr int SF = DAG ? +1 : -1;
+    const int Vs = g.Vs;
     const bool IM = mu == 0 || mu == 2;
     const bool neg = mu == 1 ? hh == 0 : mu == 2 ? hh != 0 : false;
     const int ps = mu < 2 ? 3 - hh : 2 + hh;
@@ -481,7 +482,7 @@ __device__ __forceinline__ void half_pair(int mu, const void *in, int Vs, int nf
             h[c] = cxsign(SF > 0 ? cadd(ph[c], fd) : csub(ph[c], fd), flip_f);
             if (zero_f) h[c] = C<R>{R(0), R(0)};
         }
-        LinkIO<P, RECON>::load(gf, Vs, kf, u);
+        load_link<P, RECON>(g, gf, Vs, kf, u);
         su3_mult1<false>(u, h, wf);
     }
     {
@@ -494,7 +495,7 @@ __device__ __forceinline__ void half_pair(int mu, const void *in, int Vs, int nf
             h[c] = cxsign(SF > 0 ? csub(ph[c], fd) : cadd(ph[c], fd), flip_b);
             if (zero_b) h[c] = C<R>{R(0), R(0)};
         }
-        LinkIO<P, RECON>::load(gb, Vs, kb, u);
+        load_link<P, RECON>(g, gb, Vs, kb, u);
         // sum = w_f + U^dag h
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -518,7 +519,7 @@ __device__ __forceinline__ void half_dir(const Geom &g, const void *in, const ch
     const int L = g.L[MU], st = g.stride[MU];
     const int sf = WD_IDX(g, (c == L - 1) ? s - (L - 1) * st : s + st, g.V, 1);
     const int sb = WD_IDX(g, (c == 0) ? s + (L - 1) * st : s - st, g.V, 2);
-    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(MU, in, g.Vs, sf, gdir, s, MU == 3 && g.antiperiodic && c == L - 1,
+    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(g, MU, in, sf, gdir, s, MU == 3 && g.antiperiodic && c == L - 1,
                                                 sb, gdir, sb, MU == 3 && g.antiperiodic && c == 0, hh, acc,
                                                 MU == 3 && g.split_t && c == L - 1, MU == 3 && g.split_t && c == 0);
 }
@@ -529,7 +530,7 @@ __device__ __forceinline__ void half_dir_eo(const Geom &g, const void *in, const
     const int L = g.L[MU], st = g.stride[MU];
     const int nf = WD_IDX(g, (c == L - 1) ? n - (L - 1) * st : n + st, 2 * g.V, 3);
     const int nb = WD_IDX(g, (c == 0) ? n + (L - 1) * st : n - st, 2 * g.V, 4);
-    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(MU, in, g.Vs, nf >> 1, gp, k, MU == 3 && g.antiperiodic && c == L - 1,
+    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(g, MU, in, nf >> 1, gp, k, MU == 3 && g.antiperiodic && c == L - 1,
                                                 nb >> 1, gq, nb >> 1, MU == 3 && g.antiperiodic && c == 0, hh, acc);
 }
 
@@ -730,6 +731,237 @@ template <class R> __device__ __forceinline__ void exchange_halves(C<R> (&acc)[9
     }
 }
 
+
+// ---------------------------------------------------------------- FP64 on the integer pipe
+// The FP64 hops with links and half spinors as fixed-point limbs (fixed64.cuh).  The lane's
+// eight hops share one running power-of-two unit 2^(E - 1022): a hop whose spinors are larger
+// than the unit raises it and shifts the sums down.  FP64 arithmetic remains for the final
+// sums as doubles and for what this cannot take (recon-8 links, links that are not unitary,
+// non-finite, huge or tiny spinors), which goes through half_native.
+struct FxAcc {
+    long long v[18];  // upper spin hh, lower spin 3 - hh, lower spin 2 + hh: 3 x (re, im) each
+    int E;            // the unit: 2^(E - 1022 - 57)
+    int bad;          // a spinor this arithmetic cannot take: redo the site in FP64
+};
+
+// The link's limbs; recon-12 rebuilds row 2 = conj(row0 x row1) in the same arithmetic.
+template <int RECON>
+__device__ __forceinline__ void fx_load_link(const char *gdir, int Vs, int s, int4 (&u)[9]) {
+    const int4 *p = reinterpret_cast<const int4 *>(gdir) + s;
+    constexpr int n = RECON == 12 ? 6 : 9;
+#pragma unroll
+    for (int e = 0; e < n; ++e) u[e] = __ldg(p + (size_t)e * Vs);
+    if constexpr (RECON == 12) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            // conj(a b - c d) with a = u[i], b = u[3 + j], c = u[j], d = u[3 + i]
+            const int i = (k + 1) % 3, j = (k + 2) % 3;
+            const int4 a = u[i], b = u[3 + j], c = u[j], d = u[3 + i];
+            const long long half = 1ll << (kFxBits - 1);
+            // re = a.re b.re - a.im b.im - c.re d.re + c.im d.im; im = -(a.re b.im + a.im b.re - c.re d.im - c.im d.re)
+            long long hr = fx_mac(a.x, b.x, fx_mac(-a.z, b.z, fx_mac(-c.x, d.x, fx_mac(c.z, d.z, 0))));
+            long long mr = fx_mac(a.x, b.y, fx_mac(a.y, b.x, fx_mac(-a.z, b.w, fx_mac(-a.w, b.z, half))));
+            mr = fx_mac(-c.x, d.y, fx_mac(-c.y, d.x, fx_mac(c.z, d.w, fx_mac(c.w, d.z, mr))));
+            long long hi = fx_mac(-a.x, b.z, fx_mac(-a.z, b.x, fx_mac(c.x, d.z, fx_mac(c.z, d.x, 0))));
+            long long mi = fx_mac(-a.x, b.w, fx_mac(-a.y, b.z, fx_mac(-a.z, b.y, fx_mac(-a.w, b.x, half))));
+            mi = fx_mac(c.x, d.w, fx_mac(c.y, d.z, fx_mac(c.z, d.y, fx_mac(c.w, d.x, mi))));
+            hr += mr >> kFxBits;
+            hi += mi >> kFxBits;
+            int4 o;
+            o.x = (int)((hr + half) >> kFxBits);
+            o.y = (int)hr - (int)((unsigned)o.x << kFxBits);
+            o.z = (int)((hi + half) >> kFxBits);
+            o.w = (int)hi - (int)((unsigned)o.z << kFxBits);
+            u[6 + k] = o;
+        }
+    }
+}
+
+// One hop of direction MU (ADJ: backward, U^dag) from site n with the link at sl: the half
+// spinor h = psi_hh + S f psi_ps (S the projector's sign, flip the boundary's), w = U h, then
+// upper spin += w and lower spin ps += S conj(f) w, in units of acc.E, which is raised first
+// where the spinor needs it.
+template <int RECON, bool DAG, int MU, bool ADJ, bool NC>
+__device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs, int n, int sl, int hh, bool flip,
+                                       bool zero, FxAcc &acc) {
+    constexpr bool IM = MU == 0 || MU == 2;         // f = +-i: the parts of psi_ps swap
+    constexpr int SM = DAG != ADJ ? 0 : -1;         // sign masks: of S,
+    constexpr int LO = MU < 2 ? 6 : 12;
+    const int neg = MU == 1 ? hh - 1 : MU == 2 ? -hh : 0;  // of f,
+    const int fl = MU == 3 && flip ? -1 : 0;               // of the boundary
+    const int ps = MU < 2 ? 3 - hh : 2 + hh;
+    C<double> ph[3], pd[3];
+    load_spin<F64, NC>(in, Vs, n, hh, ph);
+    load_spin<F64, NC>(in, Vs, n, ps, pd);
+    float mx = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        mx = fx_max(mx, ph[c].re, ph[c].im);
+        mx = fx_max(mx, pd[c].re, pd[c].im);
+    }
+    const int e = __float_as_int(mx) >> 20;
+    if (e > acc.E) {
+        const int sh = min(e - acc.E, 63);
+        acc.E = e;
+#pragma unroll
+        for (int k = 0; k < 18; ++k) acc.v[k] >>= sh;
+        if (e > kFxMaxExp) acc.bad = 1;
+    }
+    if (e < kFxMinExp) {
+        long long any = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            any |= __double_as_longlong(ph[c].re) | __double_as_longlong(ph[c].im) | __double_as_longlong(pd[c].re) |
+                   __double_as_longlong(pd[c].im);
+        if (any << 1) acc.bad = 1;
+    }
+    const unsigned cc = ((unsigned)(acc.E + 4) << 21) | 0x1fffffu;
+    int H[6], L[6];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        // f d: f = +-1: (re, im); f = +-i: (-im, re)
+        fx_sum(ph[c].re, fl, IM ? pd[c].im : pd[c].re, SM ^ neg ^ (IM ? -1 : 0) ^ fl, cc, H[2 * c], L[2 * c]);
+        fx_sum(ph[c].im, fl, IM ? pd[c].re : pd[c].im, SM ^ neg ^ fl, cc, H[2 * c + 1], L[2 * c + 1]);
+    }
+    if (MU == 3 && zero) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) H[k] = L[k] = 0;
+    }
+    int4 u[9];
+    fx_load_link<RECON>(gdir, Vs, sl, u);
+    const long long half = 1ll << (kFxBits - 1);
+    int XH[3], XL[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        XH[b] = H[2 * b] + H[2 * b + 1];
+        XL[b] = L[2 * b] + L[2 * b + 1];
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        // complex products on three real ones (exact sums): with P = ur x, Q = ui y and
+        // T = (ur +- ui)(x + y), u h = P - Q + i (T - P - Q) and conj(u) h = P + Q + i (T - P + Q)
+        // (T with ur - ui); high and middle sums of each
+        long long ph2 = 0, pm2 = 0, qh2 = 0, qm2 = 0, th2 = 0, tm2 = 0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int4 q = ADJ ? u[3 * b + a] : u[3 * a + b];
+            ph2 = fx_mac(q.x, H[2 * b], ph2);
+            pm2 = fx_mac(q.y, H[2 * b], fx_mac(q.x, L[2 * b], pm2));
+            qh2 = fx_mac(q.z, H[2 * b + 1], qh2);
+            qm2 = fx_mac(q.w, H[2 * b + 1], fx_mac(q.z, L[2 * b + 1], qm2));
+            const int uh = ADJ ? q.x - q.z : q.x + q.z, ul = ADJ ? q.y - q.w : q.y + q.w;
+            th2 = fx_mac(uh, XH[b], th2);
+            tm2 = fx_mac(ul, XH[b], fx_mac(uh, XL[b], tm2));
+        }
+        const long long hr = ADJ ? ph2 + qh2 : ph2 - qh2, hi = ADJ ? th2 - ph2 + qh2 : th2 - ph2 - qh2;
+        const long long mr = (ADJ ? pm2 + qm2 : pm2 - qm2) + half;
+        const long long mi = (ADJ ? tm2 - pm2 + qm2 : tm2 - pm2 - qm2) + half;
+        const long long wr = hr + (mr >> kFxBits), wi = hi + (mi >> kFxBits);
+        acc.v[2 * a] += wr;
+        acc.v[2 * a + 1] += wi;
+        // S conj(f) w: conj(f) = +-1: (re, im); conj(f) = -+i: +-(im, -re)
+        const long long m = neg;
+        const long long dr = (IM ? wi : wr) ^ m, di = (IM ? wr : wi) ^ m;
+        if (SM == 0) acc.v[LO + 2 * a] += dr - m;
+        else acc.v[LO + 2 * a] -= dr - m;
+        if ((SM == 0) != IM) acc.v[LO + 2 * a + 1] += di - m;
+        else acc.v[LO + 2 * a + 1] -= di - m;
+    }
+}
+
+// the sum of the lane's eight hops at site s (checkerboard index s with EO)
+template <int RECON, bool DAG, bool EO, bool NC>
+__device__ __forceinline__ void fx_hopping(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
+                                           int hh, FxAcc &acc) {
+    int xc[4], m = s;
+    const char *gp = reinterpret_cast<const char *>(gauge), *gq = gp;
+    if constexpr (EO) {
+        m = eo_full_index(g, s, xc[0], xc[1], xc[2], xc[3]);
+        gp += (size_t)(4 * g.eo_parity) * gdir_bytes;
+        gq += (size_t)(4 * (1 - g.eo_parity)) * gdir_bytes;
+    } else {
+        int rem = s;
+        xc[0] = rem % g.L[0]; rem /= g.L[0];
+        xc[1] = rem % g.L[1]; rem /= g.L[1];
+        xc[2] = rem % g.L[2];
+        xc[3] = rem / g.L[2];
+    }
+    auto dir = [&](auto muc) {
+        constexpr int MU = decltype(muc)::value;
+        const int L = g.L[MU], st = g.stride[MU], c = xc[MU];
+        int nf = WD_IDX(g, (c == L - 1) ? m - (L - 1) * st : m + st, EO ? 2 * g.V : g.V, EO ? 3 : 1);
+        int nb = WD_IDX(g, (c == 0) ? m + (L - 1) * st : m - st, EO ? 2 * g.V : g.V, EO ? 4 : 2);
+        if (EO) { nf >>= 1; nb >>= 1; }
+        const bool anti = MU == 3 && g.antiperiodic, cut = !EO && MU == 3 && g.split_t;
+        fx_hop<RECON, DAG, MU, false, NC>(in, gp + (size_t)MU * gdir_bytes, g.Vs, nf, s, hh, anti && c == L - 1,
+                                          cut && c == L - 1, acc);
+        fx_hop<RECON, DAG, MU, true, NC>(in, gq + (size_t)MU * gdir_bytes, g.Vs, nb, nb, hh, anti && c == 0,
+                                         cut && c == 0, acc);
+    };
+    dir(std::integral_constant<int, 0>{});
+    dir(std::integral_constant<int, 1>{});
+    dir(std::integral_constant<int, 2>{});
+    dir(std::integral_constant<int, 3>{});
+}
+
+// the same lane's sum in FP64 arithmetic, out of line: the path of what fixed point cannot take
+template <int RECON, bool DAG, bool EO, bool NC>
+__device__ __noinline__ void half_native(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
+                                         int hh, C<double> (&acc)[9]) {
+    hopping_half<F64, RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+}
+
+// The hopping sum of site s for the spins this lane owns (hh and 3 - hh), zero where `on` is
+// false.  Every lane of the warp calls it (on is the same for both lanes of a site).
+template <int P, int RECON, bool DAG, bool EO, bool NC = true>
+__device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
+                                            int hh, bool on, C<typename Real<P>::T> (&own)[6]) {
+    using R = typename Real<P>::T;
+    if constexpr (P == F64 && RECON != 8) {
+        bool native = !g.links_fx;
+        if (!native) {
+            FxAcc acc;
+#pragma unroll
+            for (int k = 0; k < 18; ++k) acc.v[k] = 0;
+            acc.E = kFxMinExp;
+            acc.bad = 0;
+            if (on) fx_hopping<RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+            // bring both lanes of the site to one unit, then complete spin 3 - hh
+            const int Ep = __shfl_xor_sync(0xffffffffu, acc.E, 16);
+            const int E = max(acc.E, Ep), sh = min(E - acc.E, 63), e = E - 1022 - kFxSpinorBits;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const long long o = __shfl_xor_sync(0xffffffffu, acc.v[12 + k] >> sh, 16);
+                const long long up = acc.v[k] >> sh, dn = (acc.v[6 + k] >> sh) + o;
+                const double a = fx_value(up, e), b = fx_value(dn, e);
+                if (k & 1) { own[k / 2].im = a; own[3 + k / 2].im = b; }
+                else { own[k / 2].re = a; own[3 + k / 2].re = b; }
+            }
+            native = acc.bad;
+        }
+        if (__any_sync(0xffffffffu, native)) {
+            native |= __shfl_xor_sync(0xffffffffu, native, 16) != 0;
+            C<double> acc[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) acc[k] = C<double>{0.0, 0.0};
+            if (on && native) half_native<RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+            exchange_halves(acc);
+            if (native)
+#pragma unroll
+                for (int k = 0; k < 6; ++k) own[k] = acc[k];
+        }
+    } else {
+        C<R> acc[9];
+        if (on) hopping_half<P, RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+        else
+#pragma unroll
+            for (int k = 0; k < 9; ++k) acc[k] = C<R>{R(0), R(0)};
+        exchange_halves(acc);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) own[k] = acc[k];
+    }
+}
+
 // The components of a site one thread owns in an epilogue: all 12, or the 6 of
 // spins hh and 3 - hh (two lanes per site).  comp(k) is the global component of
 // local component k.
@@ -796,8 +1028,10 @@ __device__ __forceinline__ void store_part(const Pt &pt, void *base, int Vs, int
 
 // Register budget: the FP32 and FP16 kernels are memory-bound and want many
 // resident warps, so they are held to 3 blocks of 256 threads per SM (at most 85
-// registers); FP64 and DF32 are arithmetic-bound and keep the compiler's choice.
-template <int P> constexpr int dslash_min_blocks() { return (P == F32 || P == F16) ? 3 : 0; }
+// registers); the fixed-point FP64 hops wait on integer results and loads and are held to
+// 128 (the compiler's 144: 1013 against 880-903 us at 32^3 x 64; 112 registers 889, 96 with
+// more spills 907); DF32 is arithmetic-bound and keeps the compiler's choice.
+template <int P> constexpr int dslash_min_blocks() { return (P == F32 || P == F16) ? 3 : P == F64 ? 2 : 0; }
 
 // Site tile (tile_x, in [0, gridDim.x)) and right-hand-side group (tile_y, in
 // [0, gridDim.y)) of this block.  Blocks start in linear order (x fastest); numbering
@@ -840,18 +1074,10 @@ __global__ void __launch_bounds__(256, dslash_min_blocks<P>()) dslash_kernel(Dsl
         for (int s0 = tile_x() * spb; s0 < a.g.V; s0 += gridDim.x * spb) {
             const int s = s0 + sl;
             const bool on = row && s < a.g.V;
-            C<R> acc[9];
-            if (on && !zin) hopping_half<P, RECON, DAG, EO>(a.g, in, a.gauge, a.gauge_dir, s, hh, acc);
-            else
-#pragma unroll
-                for (int k = 0; k < 9; ++k) acc[k] = C<R>{R(0), R(0)};
-            exchange_halves(acc);  // warp-uniform: row and s0 are the same for all 32 lanes
-            if (on) {
-                C<R> own[6];
-#pragma unroll
-                for (int k = 0; k < 6; ++k) own[k] = acc[k];
-                Ep::template site<P>(a, s, r, xin, own, st, pt);
-            }
+            C<R> own[6];
+            // all 32 lanes: row and s0 are the same for them
+            hopping_own<P, RECON, DAG, EO>(a.g, in, a.gauge, a.gauge_dir, s, hh, on && !zin, own);
+            if (on) Ep::template site<P>(a, s, r, xin, own, st, pt);
         }
     } else {
         const SiteAll pt{};

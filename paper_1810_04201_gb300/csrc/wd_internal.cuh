@@ -2,7 +2,9 @@
 //
 // Field layouts are described in include/wd.h.  Gauge layouts (per direction mu,
 // blocks of Vs sites, complex entries row-major A*3+B):
-//   F64 recon-18: 9 arrays of Vs double2            recon-12: 6 arrays (rows 0, 1)
+//   F64 recon-18: 9 arrays of Vs int4               recon-12: 6 arrays (rows 0, 1)
+//     (re.H, re.L, im.H, im.L): 58-bit fixed point, see fixed64.cuh; links that are not
+//     unitary (Geom::links_fx = 0) are kept as double2 instead
 //   F32 recon-18: 4 arrays of Vs float4 (entries 0-7) + 1 array of Vs float2 (entry 8)
 //   F32 recon-12: 3 arrays of Vs float4
 //   F16 recon-18: 2 arrays of Vs uint4 (8 half2 entries 0-7) + 1 array of Vs half2
@@ -24,6 +26,7 @@
 
 #include "../../include/wd.h"
 #include "df32.cuh"
+#include "fixed64.cuh"
 
 namespace wd {
 
@@ -80,6 +83,7 @@ struct Geom {
     unsigned *dbg;   // debug builds: the context's word for the first out-of-range index
     int split_t;     // 1: one sub-lattice of a lattice split along t; the t hops that leave it
                      // (from the first slice backward, from the last slice forward) are omitted
+    int links_fx;    // FP64 links of recon 18 and 12 are fixed-point limbs (0: doubles)
 };
 
 // Index checks of debug builds (compiled with -DWD_DEBUG, in place of a memory checker):
@@ -290,7 +294,8 @@ template <int P, int RECON> struct LinkIO;
 
 template <int RECON> struct LinkIO<F64, RECON> {
     using R = double;
-    static __device__ __forceinline__ void load(const void *dir_base, int Vs, int s, C<R> (&u)[9]) {
+    // fx: the entries are fixed-point limbs (recon 18 and 12)
+    static __device__ __forceinline__ void load(const void *dir_base, int Vs, int s, C<R> (&u)[9], bool fx) {
         const double2 *p = reinterpret_cast<const double2 *>(dir_base) + s;
         if constexpr (RECON == 8) {
 #pragma unroll
@@ -305,8 +310,13 @@ template <int RECON> struct LinkIO<F64, RECON> {
         constexpr int n = RECON == 12 ? 6 : 9;
 #pragma unroll
         for (int e = 0; e < n; ++e) {
-            double2 t = __ldg(p + (size_t)e * Vs);
-            u[e] = C<R>{t.x, t.y};
+            if (fx) {
+                const int4 t = __ldg(reinterpret_cast<const int4 *>(p) + (size_t)e * Vs);
+                u[e] = C<R>{fx_link_value(t.x, t.y), fx_link_value(t.z, t.w)};
+            } else {
+                double2 t = __ldg(p + (size_t)e * Vs);
+                u[e] = C<R>{t.x, t.y};
+            }
         }
         if (RECON == 12) rebuild_row2(u);
     }
@@ -405,6 +415,14 @@ template <int RECON> struct LinkIO<F16, RECON> {
         }
     }
 };
+
+// link of a direction in the layout of the lattice's geometry
+template <int P, int RECON>
+__device__ __forceinline__ void load_link(const Geom &g, const void *dir_base, int Vs, int s,
+                                          C<typename Real<P>::T> (&u)[9]) {
+    if constexpr (P == F64) LinkIO<P, RECON>::load(dir_base, Vs, s, u, g.links_fx != 0);
+    else LinkIO<P, RECON>::load(dir_base, Vs, s, u);
+}
 
 // ------------------------------------------------------------------ reductions
 // Deterministic block reduction of NV doubles per row of a (SB x RT) block.  SB is a

@@ -1,0 +1,99 @@
+"""The FP64 operator's fixed-point hops at the edges of their range: spinors of very different
+magnitude next to one another, zero and tiny and huge ones, and links that are not unitary
+(which go through FP64 arithmetic), against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1810_04201_gb300 import gen
+
+pytestmark = pytest.mark.gpu
+DIMS, KAPPA = (4, 3, 5, 6), 0.12
+
+
+def lattice(U, dims=DIMS, recon=18):
+    from paper_1810_04201_gb300 import wd
+    lat = wd.Lattice(dims)
+    lat.set_gauge(U, recon=recon)
+    return lat
+
+
+def apply(lat, psi, dagger=False):
+    fo = lat.new_field()
+    lat.apply(KAPPA, lat.pack(psi), fo, dagger=dagger)
+    return lat.unpack(fo)
+
+
+def neighbourhood_max(psi, dims):
+    """Largest component of each site and its eight neighbours."""
+    m = np.abs(psi.view(np.float64)).reshape(*dims[::-1], -1).max(-1)
+    out = m.copy()
+    for ax in range(4):
+        out = np.maximum(out, np.maximum(np.roll(m, 1, ax), np.roll(m, -1, ax)))
+    return out.reshape(-1)
+
+
+@pytest.mark.parametrize("recon", [18, 12])
+@pytest.mark.parametrize("decades", [0, 3, 20, 120])
+def test_magnitudes_that_differ_between_neighbours(recon, decades):
+    """Sites scaled by 10^(+-decades): each site's error is bounded by its own neighbourhood's
+    largest component (the unit of a lane is at most twice that, its resolution 2^-57: eight
+    hops of at most 16 units at |kappa| < 1, and the FP64 rounding of the oracle, stay below 2e-15)."""
+    U = gen.haar_links(DIMS, seed=3)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    s = 10.0 ** (decades * (2.0 * gen.uniform(5, gen.STREAM_MISC, 0, psi.shape[0]) - 1.0))
+    psi = psi * s[:, None, None]
+    lat = lattice(U, recon=recon)
+    for dagger in (False, True):
+        got = apply(lat, psi, dagger)
+        ref = oracle.apply_D(U, psi, KAPPA, DIMS, dagger=dagger)
+        err = np.abs(got - ref).reshape(psi.shape[0], -1).max(1)
+        assert np.all(err <= 2e-15 * neighbourhood_max(psi, DIMS))
+
+
+@pytest.mark.parametrize("scale", [1e-306, 1e-290, 1e-269, 1e-260, 1e290, 1e302, 1e304])
+def test_scales_at_the_ends_of_the_double_range(scale):
+    U = gen.haar_links(DIMS, seed=3)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    ref = oracle.apply_D(U, psi, KAPPA, DIMS)
+    got = apply(lattice(U), psi * scale)
+    # multiplying by the scale rounds; subnormal products below 1e-306 lose up to 5e-324 each
+    assert oracle.rel_err(got / scale, ref) < (1e-13 if scale > 1e-300 else 1e-12)
+
+
+def test_zeros_stay_exact():
+    """A point source reaches its neighbours and nothing else; with unit links the other
+    colours stay exactly zero."""
+    psi = gen.point_source(DIMS, 17, 2, 1)
+    got = apply(lattice(gen.haar_links(DIMS, seed=3)), psi)
+    far = neighbourhood_max(psi, DIMS) == 0
+    assert far.any() and np.all(got[far] == 0)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    psi[:, :, (0, 2)] = 0
+    got = apply(lattice(gen.unit_links(DIMS)), psi)
+    assert np.all(got[:, :, (0, 2)] == 0)
+    assert oracle.rel_err(got, oracle.apply_D(gen.unit_links(DIMS), psi, KAPPA, DIMS)) < 1e-13
+
+
+@pytest.mark.parametrize("factor", [1.0 + 2.0 ** -13, 1.01, 3.0, 1e-3])
+def test_links_that_are_not_unitary(factor):
+    U = gen.haar_links(DIMS, seed=3)
+    U[2, 7] *= factor
+    psi = gen.gaussian_source(DIMS, seed=4)
+    lat = lattice(U)
+    for dagger in (False, True):
+        assert oracle.rel_err(apply(lat, psi, dagger), oracle.apply_D(U, psi, KAPPA, DIMS, dagger=dagger)) < 1e-13
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_non_finite_spinors_reach_their_neighbours_only(bad):
+    U = gen.haar_links(DIMS, seed=3)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    psi[29, 1, 0] = bad
+    got = apply(lattice(U), psi)
+    near = ~np.isfinite(neighbourhood_max(psi, DIMS))
+    clean = psi.copy()
+    clean[29, 1, 0] = 0
+    ref = oracle.apply_D(U, clean, KAPPA, DIMS)
+    assert not np.isfinite(got[near].reshape(near.sum(), -1)).all(1).any()
+    assert oracle.rel_err(got[~near], ref[~near]) < 1e-13
