@@ -50,11 +50,28 @@ static void gauge_pack(const double *canon, void *dst, const Geom &g, size_t dir
     k_gauge_pack<P, RECON><<<grid, 128, 0, st>>>(reinterpret_cast<const double2 *>(canon), dst, g.V, g.Vs, dir, g.links_fx);
 }
 
+// *buf: a device buffer for links of compression recon (its size depends on that alone); one of
+// another compression is freed, with the graphs that hold its address
+static wd_status link_buffer(wd_ctx *c, void **buf, int *have, int recon, size_t bytes) {
+    if (*buf && *have == recon) return WD_OK;
+    if (*buf) {
+        WD_CUDA(c, cudaStreamSynchronize(c->stream));
+        cudaFree(*buf);
+        *buf = nullptr;
+        graph_clear(c);
+    }
+    WD_CUDA(c, cudaMalloc(buf, bytes));
+    *have = recon;
+    return WD_OK;
+}
+
 wd_status gauge_get(wd_ctx *c, Prec p, const void **out) {
     if (!c->has_gauge) return fail(c, WD_ERR_STATE, "no gauge field set (call wd_set_gauge first)");
-    if (!c->gauge[p]) {
-        void *d = nullptr;
-        WD_CUDA(c, cudaMalloc(&d, gauge_bytes(p, link_recon(c, p), c->g.Vs)));
+    if (!c->gauge_ok[p]) {
+        wd_status s = link_buffer(c, &c->gauge[p], &c->gauge_recon[p], link_recon(c, p),
+                                  gauge_bytes(p, link_recon(c, p), c->g.Vs));
+        if (s != WD_OK) return s;
+        void *d = c->gauge[p];
         const size_t dir = gauge_dir_bytes(c, p);
         with_recon(link_recon(c, p), [&](auto rc) {
             constexpr int R = decltype(rc)::value;
@@ -65,7 +82,7 @@ wd_status gauge_get(wd_ctx *c, Prec p, const void **out) {
         });
         WD_CUDA(c, cudaGetLastError());
         c->launches += 1;
-        c->gauge[p] = d;
+        c->gauge_ok[p] = true;
     }
     *out = c->gauge[p];
     return WD_OK;
@@ -108,7 +125,9 @@ static wd_status check_unitary(wd_ctx *c) {
     unsigned bad = 0;
     WD_CUDA(c, cudaMemcpyAsync(&bad, w, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
     WD_CUDA(c, cudaStreamSynchronize(c->stream));
-    c->g.links_fx = bad ? 0 : 1;
+    const int fx = bad ? 0 : 1;
+    if (fx != c->g.links_fx) graph_clear(c);  // graphs hold the geometry
+    c->g.links_fx = fx;
     return WD_OK;
 }
 
@@ -130,9 +149,10 @@ wd_status gauge_get_eo(wd_ctx *c, Prec p, const void **out, size_t *dir_bytes) {
     if (!c->has_gauge) return fail(c, WD_ERR_STATE, "no gauge field set (call wd_set_gauge first)");
     const int Vhs = eo_geom(c, 0).Vs;
     const size_t dir = round_up(link_dir_bytes(p, link_recon(c, p), Vhs), 256);
-    if (!c->gauge_eo[p]) {
-        void *d = nullptr;
-        WD_CUDA(c, cudaMalloc(&d, 8 * dir));
+    if (!c->gauge_eo_ok[p]) {
+        wd_status s = link_buffer(c, &c->gauge_eo[p], &c->gauge_eo_recon[p], link_recon(c, p), 8 * dir);
+        if (s != WD_OK) return s;
+        void *d = c->gauge_eo[p];
         with_recon(link_recon(c, p), [&](auto rc) {
             constexpr int R = decltype(rc)::value;
             if (p == F64) gauge_pack_eo<F64, R>(c->gauge_canon, d, c->g, Vhs, dir, c->stream);
@@ -142,7 +162,7 @@ wd_status gauge_get_eo(wd_ctx *c, Prec p, const void **out, size_t *dir_bytes) {
         });
         WD_CUDA(c, cudaGetLastError());
         c->launches += 1;
-        c->gauge_eo[p] = d;
+        c->gauge_eo_ok[p] = true;
     }
     *out = c->gauge_eo[p];
     *dir_bytes = dir;
@@ -295,24 +315,16 @@ wd_status wd_set_gauge(wd_ctx *c, const double *U, int on_device, int recon) {
     if (recon != 18 && recon != 12 && recon != 8) return fail(c, WD_ERR_ARG, "wd_set_gauge: recon must be 18, 12 or 8");
     const size_t bytes = (size_t)4 * c->g.V * 9 * 16;
     WD_CUDA(c, cudaStreamSynchronize(c->stream));
-    for (int p = 0; p < kNumPrec; ++p) {
-        if (c->gauge[p]) {
-            cudaFree(c->gauge[p]);
-            c->gauge[p] = nullptr;
-        }
-        if (c->gauge_eo[p]) {
-            cudaFree(c->gauge_eo[p]);
-            c->gauge_eo[p] = nullptr;
-        }
-    }
+    // the copies are written again when next needed, in place (16^3 x 32, new links and an FP32
+    // solve from host buffers: 4.97 ms with them freed, allocated and the solver's graph rebuilt
+    // each time, 4.57 ms without)
+    for (int p = 0; p < kNumPrec; ++p) c->gauge_ok[p] = c->gauge_eo_ok[p] = false;
     if (!c->gauge_canon) WD_CUDA(c, cudaMalloc(&c->gauge_canon, bytes));
     WD_CUDA(c, cudaMemcpyAsync(c->gauge_canon, U, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                c->stream));
     c->recon = recon;
     for (int p = 0; p < kNumPrec; ++p) c->recon_p[p] = 0;
     c->has_gauge = false;
-    // graphs bake gauge pointers in
-    graph_clear(c);
     if (recon == 8) {
         wd_status s = check_recon8(c, "wd_set_gauge");
         if (s != WD_OK) return s;
@@ -353,11 +365,8 @@ wd_status wd_set_link_compression(wd_ctx *c, wd_prec prec, int recon) {
         if (s != WD_OK) return s;
     }
     WD_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (c->gauge[prec]) cudaFree(c->gauge[prec]);
-    if (c->gauge_eo[prec]) cudaFree(c->gauge_eo[prec]);
-    c->gauge[prec] = c->gauge_eo[prec] = nullptr;
+    c->gauge_ok[prec] = c->gauge_eo_ok[prec] = false;
     c->recon_p[prec] = recon;
-    graph_clear(c);
     return WD_OK;
 }
 

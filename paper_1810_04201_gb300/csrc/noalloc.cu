@@ -56,7 +56,7 @@ extern "C" wd_status wd_normal_apply_noalloc(wd_ctx *c, double kappa, const void
         return fail(c, WD_ERR_ARG, msg);
     }
     if (!c->has_gauge) return fail(c, WD_ERR_STATE, "wd_normal_apply_noalloc: no gauge field set");
-    if (!c->gauge[prec])
+    if (!c->gauge_ok[prec])
         return fail(c, WD_ERR_STATE,
                     "wd_normal_apply_noalloc: the gauge copy in this precision does not exist (yet, or any more "
                     "after wd_set_link_compression); one wd_apply in this precision creates it (and allocates)");

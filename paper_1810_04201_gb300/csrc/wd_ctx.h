@@ -17,6 +17,11 @@ struct wd_ctx {
     bool has_gauge = false;
     void *gauge[wd::kNumPrec] = {};                    // per precision (at this->recon)
     void *gauge_eo[wd::kNumPrec] = {};                 // checkerboard copies, per precision
+    // whether a copy holds the current links, and the compression it has: new links or another
+    // compression leave the buffers (solver graphs hold their addresses) until gauge_get fills or
+    // replaces them
+    bool gauge_ok[wd::kNumPrec] = {}, gauge_eo_ok[wd::kNumPrec] = {};
+    int gauge_recon[wd::kNumPrec] = {}, gauge_eo_recon[wd::kNumPrec] = {};
     double *gauge_canon = nullptr;                     // FP64 canonical copy on device
     std::string last_error;
     long long launches = 0;

@@ -1,0 +1,55 @@
+"""Loading new links into a context that already solved: its link copies and solver graphs are
+kept and refilled, so every result must be the one a new context gives, bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1810_04201_gb300 import gen
+
+pytestmark = pytest.mark.gpu
+DIMS, KAPPA = (4, 4, 6, 8), 0.12
+
+
+def configure(lat, U, recon, inner, recon_in):
+    lat.set_gauge(U, recon=recon)
+    if recon_in != recon:
+        lat.set_link_compression(inner, recon_in)
+
+
+def results(lat, b, inner, eo):
+    fx = lat.new_field()
+    lat.cg(KAPPA, lat.pack(b), fx, tol=1e-10, inner=inner, precondition=eo)
+    fo = lat.new_field(inner)
+    lat.apply(KAPPA, lat.pack(b, inner), fo, inner)
+    return lat.unpack(fx), lat.unpack(fo, inner)
+
+
+@pytest.mark.parametrize("inner,eo", [(0, 0), (1, 0), (1, 1), (2, 1), (3, 0)])
+def test_new_links_give_what_a_new_context_gives(inner, eo):
+    from paper_1810_04201_gb300 import wd
+    U1, U2 = gen.haar_links(DIMS, seed=1), gen.haar_links(DIMS, seed=2)
+    U3 = U2.copy()
+    U3[1, 5] *= 1.0 + 2.0 ** -8  # not unitary: the FP64 links change their layout
+    b = gen.gaussian_source(DIMS, seed=3)
+    steps = [(U1, 18, 18), (U2, 18, 18), (U3, 18, 18), (U1, 18, 12), (U2, 18, 12), (U1, 12, 12), (U2, 18, 18), (U1, 8, 8)]
+    lat = wd.Lattice(DIMS)
+    for U, recon, recon_in in steps:
+        recon_in = recon if inner == 0 else recon_in
+        configure(lat, U, recon, inner, recon_in)
+        fresh = wd.Lattice(DIMS)
+        configure(fresh, U, recon, inner, recon_in)
+        for got, want in zip(results(lat, b, inner, eo), results(fresh, b, inner, eo)):
+            assert np.array_equal(got, want)
+
+
+def test_a_stale_copy_is_refused_where_a_missing_one_is():
+    from paper_1810_04201_gb300 import wd
+    lat = wd.Lattice(DIMS)
+    src = gen.gaussian_source(DIMS, seed=3)
+    for seed in (1, 2):
+        lat.set_gauge(gen.haar_links(DIMS, seed=seed))
+        f, o = lat.pack(src, 1), lat.new_field(1)
+        with pytest.raises(wd.WDError) as e:
+            lat.normal_apply_noalloc(KAPPA, f, o, 1)
+        assert e.value.status == 8
+        lat.apply(KAPPA, f, o, 1)
+        lat.normal_apply_noalloc(KAPPA, f, o, 1)
