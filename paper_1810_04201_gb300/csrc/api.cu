@@ -275,6 +275,8 @@ wd_status wd_create(wd_ctx **out, const int dims[4], int antiperiodic_t, void *s
     c->g.stride[1] = dims[0];
     c->g.stride[2] = dims[0] * dims[1];
     c->g.stride[3] = dims[0] * dims[1] * dims[2];
+    for (int mu = 0; mu < 3; ++mu) c->g.div[mu] = fast_div(dims[mu]);
+    c->g.divh = fast_div(dims[0] / 2);
     c->g.antiperiodic = antiperiodic_t ? 1 : 0;
     c->g.eo_parity = -1;
     c->g.dbg = nullptr;

@@ -273,22 +273,16 @@ template <int P, int RECON> __global__ void k_gauge_pack_eo(const double2 *canon
                                                             size_t dir_bytes) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x, mu = blockIdx.y;
     if (n >= g.V) return;
-    int rem = n;
-    const int x = rem % g.L[0]; rem /= g.L[0];
-    const int y = rem % g.L[1]; rem /= g.L[1];
-    const int z = rem % g.L[2];
-    const int t = rem / g.L[2];
+    int x, y, z, t;
+    site_xyzt(g, n, x, y, z, t);
     const int par = (x + y + z + t) & 1;
     char *base = reinterpret_cast<char *>(dst) + (size_t)(4 * par + mu) * dir_bytes;
     pack_link<P, RECON>(canon + ((size_t)mu * g.V + n) * 9, base, Vhs, n >> 1, g.links_fx != 0);
 }
 
 __device__ __forceinline__ int site_parity(const Geom &g, int n) {
-    int rem = n;
-    const int x = rem % g.L[0]; rem /= g.L[0];
-    const int y = rem % g.L[1]; rem /= g.L[1];
-    const int z = rem % g.L[2];
-    const int t = rem / g.L[2];
+    int x, y, z, t;
+    site_xyzt(g, n, x, y, z, t);
     return (x + y + z + t) & 1;
 }
 

@@ -194,7 +194,10 @@ __device__ __forceinline__ float load_raw_h2(const void *base, int Vs, int s, h2
     return ldx<NC>(SpinorIO<F16>::norms(base, Vs) + s);
 }
 
-// the 9 link entries as half2 (recon-12/8 rows are rebuilt in FP32 and rounded to half)
+// the 9 link entries as half2 (recon-12/8 rows are rebuilt in FP32 and rounded to half).
+// recon-12: row 2 = conj(row0 x row1) on the half entries themselves (products exact in FP32
+// sums), about 40 instructions a link against 75 with the entries converted to FP32 and back,
+// in a kernel bound by issue: 32^3 x 64 145.0 -> 136.9 us.
 template <int RECON>
 __device__ __forceinline__ void load_link_h2(const char *gdir, int Vs, int s, h2 (&u)[9]) {
     if constexpr (RECON == 18) {
@@ -203,6 +206,22 @@ __device__ __forceinline__ void load_link_h2(const char *gdir, int Vs, int s, h2
         u[0] = a.x; u[1] = a.y; u[2] = a.z; u[3] = a.w;
         u[4] = b.x; u[5] = b.y; u[6] = b.z; u[7] = b.w;
         u[8] = __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint4 *>(gdir) + (size_t)2 * Vs) + s);
+    } else if constexpr (RECON == 12) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(gdir) + s);
+        const uint2 b = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint4 *>(gdir) + Vs) + s);
+        u[0] = a.x; u[1] = a.y; u[2] = a.z; u[3] = a.w;
+        u[4] = b.x; u[5] = b.y;
+        h2 n[3];  // row 1 with its imaginary halves negated
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n[k] = u[3 + k] ^ 0x80000000u;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int i = (k + 1) % 3, j = (k + 2) % 3;
+            C<float> t{0.f, 0.f};
+            cmac_h(t, u[i], u[3 + j], n[j]);
+            cmac_h(t, h2_neg(u[j]), u[3 + i], n[i]);
+            u[6 + k] = f2h(t.re, -t.im);
+        }
     } else {
         C<float> w[9];
         LinkIO<F16, RECON>::load(gdir, Vs, s, w);
@@ -293,11 +312,18 @@ __device__ __forceinline__ void hopping(const Geom &g, const void *in, const voi
     using R = typename Real<P>::T;
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = C<R>{R(0), R(0)};
-    int rem = s;
-    const int x = rem % g.L[0]; rem /= g.L[0];
-    const int y = rem % g.L[1]; rem /= g.L[1];
-    const int z = rem % g.L[2];
-    const int t = rem / g.L[2];
+    int x, y, z, t;
+    if constexpr (P == F32 && RECON == 18) {
+        // HBM-bound, and the compiler's schedule with the multiplications is no faster (32^3 x 64:
+        // 196 us with divisions, 199 without; FP16 134.8 and 128.6, FP32 recon-12 169.6 and 165.5)
+        int rem = s;
+        x = rem % g.L[0]; rem /= g.L[0];
+        y = rem % g.L[1]; rem /= g.L[1];
+        z = rem % g.L[2];
+        t = rem / g.L[2];
+    } else {
+        site_xyzt(g, s, x, y, z, t);
+    }
     const char *gb = reinterpret_cast<const char *>(gauge);
     if constexpr (HasScale<P>::value) {
         hop_dir_scaled<P, RECON, DAG, 0, NC>(g, in, gb, s, x, acc);
@@ -320,13 +346,11 @@ __device__ __forceinline__ void hopping(const Geom &g, const void *in, const voi
 // backward hop reads U_mu(n - mu) at the neighbour's index.  gauge points to
 // parity 0; parity 1 follows 4 * gdir_bytes later.
 __device__ __forceinline__ int eo_full_index(const Geom &g, int k, int &x, int &y, int &z, int &t) {
-    const int lxh = g.L[0] >> 1;
-    int r = k / lxh;
-    const int xh = k - r * lxh;
-    y = r % g.L[1];
-    r /= g.L[1];
-    z = r % g.L[2];
-    t = r / g.L[2];
+    const int q = fdiv(k, g.divh), r = fdiv(q, g.div[1]);
+    const int xh = k - q * (g.L[0] >> 1);
+    y = q - r * g.L[1];
+    t = fdiv(r, g.div[2]);
+    z = r - t * g.L[2];
     x = 2 * xh + ((g.eo_parity + y + z + t) & 1);
     return WD_IDX(g, x + g.stride[1] * y + g.stride[2] * z + g.stride[3] * t, 2 * g.V, 5);
 }
@@ -676,11 +700,7 @@ __device__ __forceinline__ void hopping_half(const Geom &g, const void *in, cons
             gp += (size_t)(4 * g.eo_parity) * gdir_bytes;
             gq += (size_t)(4 * (1 - g.eo_parity)) * gdir_bytes;
         } else {
-            int rem = s;
-            xc[0] = rem % g.L[0]; rem /= g.L[0];
-            xc[1] = rem % g.L[1]; rem /= g.L[1];
-            xc[2] = rem % g.L[2];
-            xc[3] = rem / g.L[2];
+            site_xyzt(g, s, xc[0], xc[1], xc[2], xc[3]);
         }
         cd2 a9[9];
 #pragma unroll
@@ -704,11 +724,8 @@ __device__ __forceinline__ void hopping_half(const Geom &g, const void *in, cons
         half_dir_eo<P, RECON, DAG, 2, NC>(g, in, gp + 2 * gdir_bytes, gq + 2 * gdir_bytes, s, n, z, hh, acc);
         half_dir_eo<P, RECON, DAG, 3, NC>(g, in, gp + 3 * gdir_bytes, gq + 3 * gdir_bytes, s, n, t, hh, acc);
     } else {
-        int rem = s;
-        const int x = rem % g.L[0]; rem /= g.L[0];
-        const int y = rem % g.L[1]; rem /= g.L[1];
-        const int z = rem % g.L[2];
-        const int t = rem / g.L[2];
+        int x, y, z, t;
+        site_xyzt(g, s, x, y, z, t);
         const char *gb = reinterpret_cast<const char *>(gauge);
         half_dir<P, RECON, DAG, 0, NC>(g, in, gb, s, x, hh, acc);
         half_dir<P, RECON, DAG, 1, NC>(g, in, gb + gdir_bytes, s, y, hh, acc);
@@ -880,11 +897,7 @@ __device__ __forceinline__ void fx_hopping(const Geom &g, const void *in, const 
         gp += (size_t)(4 * g.eo_parity) * gdir_bytes;
         gq += (size_t)(4 * (1 - g.eo_parity)) * gdir_bytes;
     } else {
-        int rem = s;
-        xc[0] = rem % g.L[0]; rem /= g.L[0];
-        xc[1] = rem % g.L[1]; rem /= g.L[1];
-        xc[2] = rem % g.L[2];
-        xc[3] = rem / g.L[2];
+        site_xyzt(g, s, xc[0], xc[1], xc[2], xc[3]);
     }
     auto dir = [&](auto muc) {
         constexpr int MU = decltype(muc)::value;
@@ -1191,11 +1204,8 @@ __global__ void __launch_bounds__(256, K == 2 ? 2 : 1) dslash_multi_kernel(Dslas
     for (int s0 = tile_x() * blockDim.x; s0 < a.g.V; s0 += gridDim.x * blockDim.x) {
         const int s = s0 + threadIdx.x;
         if (s >= a.g.V) continue;
-        int rem = s;
-        const int x = rem % a.g.L[0]; rem /= a.g.L[0];
-        const int y = rem % a.g.L[1]; rem /= a.g.L[1];
-        const int z = rem % a.g.L[2];
-        const int t = rem / a.g.L[2];
+        int x, y, z, t;
+        site_xyzt(a.g, s, x, y, z, t);
         C<float> acc[K][12];
 #pragma unroll
         for (int k = 0; k < K; ++k)

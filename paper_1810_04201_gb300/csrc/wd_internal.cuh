@@ -73,11 +73,27 @@ template <class R> __device__ __forceinline__ C<R> cmacc(C<R> s, C<R> a, C<R> b)
 }
 
 // ------------------------------------------------------------------ geometry
+// Division of 0 <= n < 2^31 by a lattice extent d as a multiplication: with l = ceil(log2 d) and
+// mul = floor(2^(31 + l) / d) + 1, n / d = (n mul) >> (31 + l) exactly (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994).  The three divisions that give a
+// site's coordinates cost about 20 instructions each as divisions, a tenth of an FP16 site.
+struct FastDiv {
+    unsigned mul, sh;
+};
+inline FastDiv fast_div(int d) {
+    unsigned l = 0;
+    while ((1ll << l) < d) ++l;
+    return FastDiv{(unsigned)((1ull << (31 + l)) / (unsigned)d + 1), l};
+}
+__device__ __forceinline__ int fdiv(int n, FastDiv f) { return (int)(__umulhi(2u * (unsigned)n, f.mul) >> f.sh); }
+
 struct Geom {
     int L[4];
     int V;           // output sites of a launch (V, or V/2 on one parity)
     int Vs;          // site stride of field arrays (V rounded up to kSiteAlign)
     int stride[4];   // 1, Lx, Lx*Ly, Lx*Ly*Lz (full-lattice strides)
+    FastDiv div[3];  // by Lx, Ly, Lz
+    FastDiv divh;    // by Lx / 2 (checkerboards)
     int antiperiodic;
     int eo_parity;   // -1: full lattice; 0 / 1: checkerboard fields, output on this parity
     unsigned *dbg;   // debug builds: the context's word for the first out-of-range index
@@ -85,6 +101,15 @@ struct Geom {
                      // (from the first slice backward, from the last slice forward) are omitted
     int links_fx;    // FP64 links of recon 18 and 12 are fixed-point limbs (0: doubles)
 };
+
+// coordinates of site n of the full lattice
+__device__ __forceinline__ void site_xyzt(const Geom &g, int n, int &x, int &y, int &z, int &t) {
+    const int q = fdiv(n, g.div[0]), r = fdiv(q, g.div[1]);
+    t = fdiv(r, g.div[2]);
+    x = n - q * g.L[0];
+    y = q - r * g.L[1];
+    z = r - t * g.L[2];
+}
 
 // Index checks of debug builds (compiled with -DWD_DEBUG, in place of a memory checker):
 // an index outside [0, n) is recorded in the context's debug word, the first one only, as
