@@ -198,9 +198,18 @@ void graph_clear(wd_ctx *c) {
     c->graph_used.clear();
 }
 
+// Where no autotuner or wd_set_tiles chose a shape, the fused kernels take up to four right-hand
+// sides per block (12 rows of FP32 at 24^3 x 48: 128.9 ms a solve against 129.8 with one and
+// 130.8 with two per block; the plain operators differ, see tiles_for).
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
-    return it != c->cg_tiles.end() ? it->second : tiles_for(c, p, nrhs);
+    if (it != c->cg_tiles.end()) return it->second;
+    it = c->tiles.find(p * 64 + nrhs);
+    if (it != c->tiles.end()) return it->second;
+    DslashTiles t;
+    t.site_tile = 64;
+    t.rhs_tile = nrhs < 4 ? nrhs : 4;
+    return t;
 }
 
 void ws_release(wd_ctx *c, const std::string &name) {
@@ -212,12 +221,22 @@ void ws_release(wd_ctx *c, const std::string &name) {
     c->ws_size.erase(name);
 }
 
+// The launch shape where neither wd_set_tiles nor an autotuner chose one.  One right-hand side
+// per block: the blocks of a site tile's right-hand sides start together and share its links
+// through L2, and a block's rows leave no idle threads when nrhs is odd (24^3 x 48, 64 x 1
+// against 64 x 4, us: FP32 12 rows 586 / 618, 7 rows 339 / 388; FP16 408 / 438, 241 / 277).
+// FP32 rows in pairs on one thread from 2^17 site-rows on (12 rows 562, 4 rows 186 / 200; at
+// 8^3 x 16 with two rows 8.5 / 6.7).  Larger blocks for FP64 from 2^18 site-rows on (256 / 64
+// threads: 12 rows 3144 / 3289, one row at 32^3 x 64 838 / 876, at 16^4 38.6 / 36.4) and DF32
+// (128 / 64: 2810 / 2861).
 DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs) {
     auto it = c->tiles.find(p * 64 + nrhs);
     if (it != c->tiles.end()) return it->second;
+    const long long work = (long long)c->g.V * nrhs;
     DslashTiles t;
-    t.site_tile = 64;
-    t.rhs_tile = nrhs < 4 ? nrhs : 4;
+    t.site_tile = p == DF32 ? 128 : p == F64 && work >= (1 << 18) ? 256 : 64;
+    t.rhs_tile = 1;
+    if (p == F32 && nrhs % 2 == 0 && work >= (1 << 17) && !c->split) t.rhs_tile = t.rhs_per_thread = 2;
     return t;
 }
 

@@ -130,6 +130,10 @@ wd_status wd_set_rhs_per_thread(wd_ctx *c, wd_prec prec, int nrhs, int k) {
     if ((int)prec < 0 || (int)prec >= kNumPrec || nrhs < 1 || nrhs > WD_MAX_RHS || k < 1 || k > 4)
         return fail(c, WD_ERR_ARG, "wd_set_rhs_per_thread: bad argument");
     DslashTiles t = tiles_for(c, (Prec)prec, nrhs);
+    if (!c->tiles.count((int)prec * 64 + nrhs)) {  // no shape chosen yet: k of up to four rows of a block
+        t.site_tile = 64;
+        t.rhs_tile = nrhs < 4 ? nrhs : 4;
+    }
     if (k > 1 && (prec != WD_F32 || t.rhs_tile % k != 0 || (t.site_tile * t.rhs_tile / k) % 32 != 0))
         return fail(c, WD_ERR_ARG, "wd_set_rhs_per_thread: FP32 only, k dividing rhs_tile, a multiple of 32 threads");
     if (k > 1 && c->split)

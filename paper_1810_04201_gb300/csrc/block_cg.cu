@@ -252,7 +252,7 @@ template <int RECON>
 static void record_block(wd_ctx *c, double kappa, int k, const void *g64, const BlockBufs &f,
                          cudaGraphConditionalHandle hw, Plan &plan) {
     const size_t fs = spinor_bytes(F64, c->g.Vs);
-    const DslashTiles t64 = tiles_for(c, F64, k);
+    const DslashTiles t64 = cg_tiles_for(c, F64, k, false);
     DslashArgs base{};
     base.g = c->g;
     base.gauge = g64;
@@ -353,7 +353,7 @@ wd_status block_cg_solve(wd_ctx *c, double kappa, const void *b, void *x, const 
     BlockState *bs = f.bs;
     void *B = f.B, *X = f.X;
 
-    const DslashTiles t64 = tiles_for(c, F64, k);
+    const DslashTiles t64 = cg_tiles_for(c, F64, k, false);
     char key[200];
     snprintf(key, sizeof key, "bcg|%d|%d|%a|%d,%d", k, link_recon(c, F64), kappa, t64.site_tile, t64.rhs_tile);
     cudaGraphExec_t exec = (cudaGraphExec_t)graph_get(c, key);

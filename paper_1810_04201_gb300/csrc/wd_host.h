@@ -104,7 +104,7 @@ Geom eo_geom(const wd_ctx *c, int parity);
 
 DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs);
 // launch shape of the solvers' fused Dslash kernels, for plain or even-odd solves:
-// wd_autotune_cg's choice, else tiles_for
+// wd_autotune_cg's choice, else the one chosen for the plain operators, else the default
 constexpr int kEoTileKey = 1024;
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo);
 // frees a workspace buffer (no-op when absent)
