@@ -73,8 +73,8 @@ typedef enum wd_status {
 
 /* Storage and arithmetic precision of a field and of the operator applied to it.
  *   WD_F64   IEEE double.  For unitary links whole or as recon 12 the products U psi are
- *            formed in 58-bit fixed point relative to the largest neighbouring component
- *            (relative error of the operator as with IEEE arithmetic, 1.5e-16); other links,
+ *            formed from integer and FP32 parts relative to the largest neighbouring component
+ *            (the operator's relative error is no larger than with IEEE arithmetic); other links,
  *            recon 8 and spinors beyond 2^-894 .. 2^1007 use IEEE arithmetic throughout.
  *   WD_F32   IEEE single.
  *   WD_F16   half-precision storage with a per-site FP32 scale, FP32 accumulation:

@@ -146,7 +146,7 @@ template <int P> __global__ void k_zero(VecArgs v) {
 
 // One link, canonical complex128 u[9] -> the layout of precision P and recon R,
 // at index idx of arrays with stride Vs starting at `base` (one direction).
-// fx (FP64, recon 18 and 12): as fixed-point limbs.
+// fx (FP64, recon 18 and 12): as integer and float limbs.
 template <int P, int RECON>
 __device__ __forceinline__ void pack_link(const double2 *u, char *base, int Vs, int idx, bool fx) {
     if constexpr (RECON == 8) {
@@ -229,7 +229,7 @@ template <int P, int RECON> __global__ void k_gauge_pack(const double2 *canon, v
 }
 
 // *bad = 1 when the rows of some link are not orthonormal to 2^-11 (NaN included): the
-// fixed-point FP64 arithmetic needs unitary links (fixed64.cuh)
+// FP64 products on limbs need unitary links (fixed64.cuh)
 template <int DUMMY = 0> __global__ void k_gauge_not_unitary(const double2 *canon, size_t nlinks, unsigned *bad) {
     for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += (size_t)gridDim.x * blockDim.x) {
         float2 u[9];

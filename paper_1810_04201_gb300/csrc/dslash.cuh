@@ -749,19 +749,21 @@ template <class R> __device__ __forceinline__ void exchange_halves(C<R> (&acc)[9
 }
 
 
-// ---------------------------------------------------------------- FP64 on the integer pipe
-// The FP64 hops with links and half spinors as fixed-point limbs (fixed64.cuh).  The lane's
-// eight hops share one running power-of-two unit 2^(E - 1022): a hop whose spinors are larger
-// than the unit raises it and shifts the sums down.  FP64 arithmetic remains for the final
-// sums as doubles and for what this cannot take (recon-8 links, links that are not unitary,
-// non-finite, huge or tiny spinors), which goes through half_native.
+// ---------------------------------------------------------------- FP64 off the FP64 pipe
+// The FP64 hops on integers and floats (fixed64.cuh).  The lane's eight hops share one running
+// power-of-two unit 2^(E - 1022): a hop whose spinors are larger than the unit raises it and
+// shifts the sums down.  The directions of a lower spin that goes to the partner lane come
+// first, so that a lane holds two spins of sums and not three.  FP64 arithmetic remains for half
+// of the projections, the final sums as doubles and for what this cannot take (recon-8 links,
+// links that are not unitary, non-finite, huge or tiny spinors), which goes through half_native.
 struct FxAcc {
-    long long v[18];  // upper spin hh, lower spin 3 - hh, lower spin 2 + hh: 3 x (re, im) each
-    int E;            // the unit: 2^(E - 1022 - 57)
+    long long v[12];  // upper spin hh, then the lower spin under way: 3 x (re, im) each
+    int E;            // the unit: 2^(E - 1022 - kFxAccBits)
     int bad;          // a spinor this arithmetic cannot take: redo the site in FP64
 };
 
-// The link's limbs; recon-12 rebuilds row 2 = conj(row0 x row1) in the same arithmetic.
+// The link's entries (re.H, re.L, im.H, im.L); recon-12 rebuilds row 2 = conj(row0 x row1) in
+// the same arithmetic.
 template <int RECON>
 __device__ __forceinline__ void fx_load_link(const char *gdir, int Vs, int s, int4 (&u)[9]) {
     const int4 *p = reinterpret_cast<const int4 *>(gdir) + s;
@@ -774,36 +776,40 @@ __device__ __forceinline__ void fx_load_link(const char *gdir, int Vs, int s, in
             // conj(a b - c d) with a = u[i], b = u[3 + j], c = u[j], d = u[3 + i]
             const int i = (k + 1) % 3, j = (k + 2) % 3;
             const int4 a = u[i], b = u[3 + j], c = u[j], d = u[3 + i];
-            const long long half = 1ll << (kFxBits - 1);
-            // re = a.re b.re - a.im b.im - c.re d.re + c.im d.im; im = -(a.re b.im + a.im b.re - c.re d.im - c.im d.re)
-            long long hr = fx_mac(a.x, b.x, fx_mac(-a.z, b.z, fx_mac(-c.x, d.x, fx_mac(c.z, d.z, 0))));
-            long long mr = fx_mac(a.x, b.y, fx_mac(a.y, b.x, fx_mac(-a.z, b.w, fx_mac(-a.w, b.z, half))));
-            mr = fx_mac(-c.x, d.y, fx_mac(-c.y, d.x, fx_mac(c.z, d.w, fx_mac(c.w, d.z, mr))));
-            long long hi = fx_mac(-a.x, b.z, fx_mac(-a.z, b.x, fx_mac(c.x, d.z, fx_mac(c.z, d.x, 0))));
-            long long mi = fx_mac(-a.x, b.w, fx_mac(-a.y, b.z, fx_mac(-a.z, b.y, fx_mac(-a.w, b.x, half))));
-            mi = fx_mac(c.x, d.w, fx_mac(c.y, d.z, fx_mac(c.z, d.y, fx_mac(c.w, d.x, mi))));
-            hr += mr >> kFxBits;
-            hi += mi >> kFxBits;
-            int4 o;
-            o.x = (int)((hr + half) >> kFxBits);
-            o.y = (int)hr - (int)((unsigned)o.x << kFxBits);
-            o.z = (int)((hi + half) >> kFxBits);
-            o.w = (int)hi - (int)((unsigned)o.z << kFxBits);
-            u[6 + k] = o;
+            long long hr = 0, hi = 0;
+            float fr = 0.f, fi = 0.f;
+            fx_cmac<false>(a, b.x, -b.z, b.z, b.x, (float)b.x, (float)b.z, __int_as_float(b.y), __int_as_float(b.w), hr, hi, fr, fi);
+            long long gr = 0, gi = 0;
+            float er = 0.f, ei = 0.f;
+            fx_cmac<false>(c, d.x, -d.z, d.z, d.x, (float)d.x, (float)d.z, __int_as_float(d.y), __int_as_float(d.w), gr, gi, er, ei);
+            const int2 re = fx_link_of(hr - gr, fr - er), im = fx_link_of(gi - hi, ei - fi);
+            u[6 + k] = make_int4(re.x, re.y, im.x, im.y);
         }
     }
 }
 
+
+// the sums in the larger unit of exponent e
+__device__ __forceinline__ void fx_raise(FxAcc &acc, int e) {
+    const int sh = min(e - acc.E, 63);
+    acc.E = e;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc.v[k] >>= sh;
+}
+
 // One hop of direction MU (ADJ: backward, U^dag) from site n with the link at sl: the half
 // spinor h = psi_hh + S f psi_ps (S the projector's sign, flip the boundary's), w = U h, then
-// upper spin += w and lower spin ps += S conj(f) w, in units of acc.E, which is raised first
-// where the spinor needs it.
+// upper spin += w and lower spin ps += S conj(|f|) w (|f| stands for i where f = +-i; the caller
+// gives the lower spin f's sign), in units of acc.E, which is raised first where the spinor needs
+// it.  Forward hops add the two spins in FP64 and convert the sum, backward hops convert both and
+// add integers: that splits the work between the FP64 pipe and the integer ones (32^3 x 64: 811-850
+// us; all on integers 876, all in FP64 870).
 template <int RECON, bool DAG, int MU, bool ADJ, bool NC>
 __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs, int n, int sl, int hh, bool flip,
                                        bool zero, FxAcc &acc) {
     constexpr bool IM = MU == 0 || MU == 2;         // f = +-i: the parts of psi_ps swap
     constexpr int SM = DAG != ADJ ? 0 : -1;         // sign masks: of S,
-    constexpr int LO = MU < 2 ? 6 : 12;
+    constexpr int LO = 6;
     const int neg = MU == 1 ? hh - 1 : MU == 2 ? -hh : 0;  // of f,
     const int fl = MU == 3 && flip ? -1 : 0;               // of the boundary
     const int ps = MU < 2 ? 3 - hh : 2 + hh;
@@ -816,12 +822,10 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
         mx = fx_max(mx, ph[c].re, ph[c].im);
         mx = fx_max(mx, pd[c].re, pd[c].im);
     }
-    const int e = __float_as_int(mx) >> 20;
+    // + 1: components stay below (1 - 2^-21) units, so that rounded limbs cannot overflow
+    const int e = (int)((__float_as_uint(mx) + 1u) >> 20);
     if (e > acc.E) {
-        const int sh = min(e - acc.E, 63);
-        acc.E = e;
-#pragma unroll
-        for (int k = 0; k < 18; ++k) acc.v[k] >>= sh;
+        fx_raise(acc, e);
         if (e > kFxMaxExp) acc.bad = 1;
     }
     if (e < kFxMinExp) {
@@ -832,62 +836,67 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
                    __double_as_longlong(pd[c].im);
         if (any << 1) acc.bad = 1;
     }
-    const unsigned cc = ((unsigned)(acc.E + 4) << 21) | 0x1fffffu;
-    int H[6], L[6];
+    const unsigned cc = ((unsigned)(acc.E + 2) << 21) | 0x1fffffu;
+    int H[6];
+    float L[6];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         // f d: f = +-1: (re, im); f = +-i: (-im, re)
-        fx_sum(ph[c].re, fl, IM ? pd[c].im : pd[c].re, SM ^ neg ^ (IM ? -1 : 0) ^ fl, cc, H[2 * c], L[2 * c]);
-        fx_sum(ph[c].im, fl, IM ? pd[c].re : pd[c].im, SM ^ neg ^ fl, cc, H[2 * c + 1], L[2 * c + 1]);
+        const double ar = IM ? pd[c].im : pd[c].re, ai = IM ? pd[c].re : pd[c].im;
+        const int mr = SM ^ neg ^ (IM ? -1 : 0), mi = SM ^ neg;
+        if constexpr (!ADJ) {
+            fx_limbs(ph[c].re + xsign(ar, mr != 0), fl, cc, H[2 * c], L[2 * c]);
+            fx_limbs(ph[c].im + xsign(ai, mi != 0), fl, cc, H[2 * c + 1], L[2 * c + 1]);
+        } else {
+            fx_sum(ph[c].re, fl, ar, mr ^ fl, cc, H[2 * c], L[2 * c]);
+            fx_sum(ph[c].im, fl, ai, mi ^ fl, cc, H[2 * c + 1], L[2 * c + 1]);
+        }
     }
     if (MU == 3 && zero) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) H[k] = L[k] = 0;
+        for (int k = 0; k < 6; ++k) {
+            H[k] = 0;
+            L[k] = 0.f;
+        }
     }
     int4 u[9];
     fx_load_link<RECON>(gdir, Vs, sl, u);
-    const long long half = 1ll << (kFxBits - 1);
-    int XH[3], XL[3];
+    float F[6];
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        XH[b] = H[2 * b] + H[2 * b + 1];
-        XL[b] = L[2 * b] + L[2 * b + 1];
-    }
+    for (int k = 0; k < 6; ++k) F[k] = (float)H[k];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        // complex products on three real ones (exact sums): with P = ur x, Q = ui y and
-        // T = (ur +- ui)(x + y), u h = P - Q + i (T - P - Q) and conj(u) h = P + Q + i (T - P + Q)
-        // (T with ur - ui); high and middle sums of each
-        long long ph2 = 0, pm2 = 0, qh2 = 0, qm2 = 0, th2 = 0, tm2 = 0;
+        long long hr = kFxHalfAcc, hi = kFxHalfAcc;
+        float fr = 0.f, fi = 0.f;
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const int4 q = ADJ ? u[3 * b + a] : u[3 * a + b];
-            ph2 = fx_mac(q.x, H[2 * b], ph2);
-            pm2 = fx_mac(q.y, H[2 * b], fx_mac(q.x, L[2 * b], pm2));
-            qh2 = fx_mac(q.z, H[2 * b + 1], qh2);
-            qm2 = fx_mac(q.w, H[2 * b + 1], fx_mac(q.z, L[2 * b + 1], qm2));
-            const int uh = ADJ ? q.x - q.z : q.x + q.z, ul = ADJ ? q.y - q.w : q.y + q.w;
-            th2 = fx_mac(uh, XH[b], th2);
-            tm2 = fx_mac(ul, XH[b], fx_mac(uh, XL[b], tm2));
+            const int x = H[2 * b], y = H[2 * b + 1];
+            fx_cmac<ADJ>(ADJ ? u[3 * b + a] : u[3 * a + b], x, ADJ ? y : -y, y, ADJ ? -x : x, F[2 * b], F[2 * b + 1],
+                         L[2 * b], L[2 * b + 1], hr, hi, fr, fi);
         }
-        const long long hr = ADJ ? ph2 + qh2 : ph2 - qh2, hi = ADJ ? th2 - ph2 + qh2 : th2 - ph2 - qh2;
-        const long long mr = (ADJ ? pm2 + qm2 : pm2 - qm2) + half;
-        const long long mi = (ADJ ? tm2 - pm2 + qm2 : tm2 - pm2 - qm2) + half;
-        const long long wr = hr + (mr >> kFxBits), wi = hi + (mi >> kFxBits);
+        const long long wr = (hr >> kFxAccShift) + __float2int_rn(fr * kFxSmallToAcc);
+        const long long wi = (hi >> kFxAccShift) + __float2int_rn(fi * kFxSmallToAcc);
         acc.v[2 * a] += wr;
         acc.v[2 * a + 1] += wi;
-        // S conj(f) w: conj(f) = +-1: (re, im); conj(f) = -+i: +-(im, -re)
-        const long long m = neg;
-        const long long dr = (IM ? wi : wr) ^ m, di = (IM ? wr : wi) ^ m;
-        if (SM == 0) acc.v[LO + 2 * a] += dr - m;
-        else acc.v[LO + 2 * a] -= dr - m;
-        if ((SM == 0) != IM) acc.v[LO + 2 * a + 1] += di - m;
-        else acc.v[LO + 2 * a + 1] -= di - m;
+        // S conj(|f|) w: conj(f) = 1: (re, im); conj(i): (im, -re)
+        constexpr bool rp = SM == 0, ip = (SM == 0) != IM;
+        if (rp) acc.v[LO + 2 * a] += IM ? wi : wr;
+        else acc.v[LO + 2 * a] -= IM ? wi : wr;
+        if (ip) acc.v[LO + 2 * a + 1] += IM ? wr : wi;
+        else acc.v[LO + 2 * a + 1] -= IM ? wr : wi;
     }
 }
 
-// the sum of the lane's eight hops at site s (checkerboard index s with EO)
-template <int RECON, bool DAG, bool EO, bool NC>
+// lower spin times -1 where m = -1
+__device__ __forceinline__ void fx_negate_lower(FxAcc &acc, int m) {
+#pragma unroll
+    for (int k = 6; k < 12; ++k) acc.v[k] = (acc.v[k] ^ (long long)m) - m;
+}
+
+// The lane's hops at site s (checkerboard index s with EO) of mu = 2, 3 (PAIR 1: the lower spin is
+// 2 + hh), then, with the partner's lower spin, which is 3 - hh here, of mu = 0, 1 (PAIR 0).  f is
+// -i for mu = 2, hh = 1 and -1 for mu = 1, hh = 0.
+template <int RECON, bool DAG, bool EO, bool NC, int PAIR>
 __device__ __forceinline__ void fx_hopping(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                            int hh, FxAcc &acc) {
     int xc[4], m = s;
@@ -911,13 +920,19 @@ __device__ __forceinline__ void fx_hopping(const Geom &g, const void *in, const 
         fx_hop<RECON, DAG, MU, true, NC>(in, gq + (size_t)MU * gdir_bytes, g.Vs, nb, nb, hh, anti && c == 0,
                                          cut && c == 0, acc);
     };
-    dir(std::integral_constant<int, 0>{});
-    dir(std::integral_constant<int, 1>{});
-    dir(std::integral_constant<int, 2>{});
-    dir(std::integral_constant<int, 3>{});
+    if constexpr (PAIR == 1) {
+        dir(std::integral_constant<int, 2>{});
+        fx_negate_lower(acc, -hh);
+        dir(std::integral_constant<int, 3>{});
+    } else {
+        fx_negate_lower(acc, hh - 1);
+        dir(std::integral_constant<int, 1>{});
+        fx_negate_lower(acc, hh - 1);
+        dir(std::integral_constant<int, 0>{});
+    }
 }
 
-// the same lane's sum in FP64 arithmetic, out of line: the path of what fixed point cannot take
+// the same lane's sum in FP64 arithmetic, out of line: the path of what limbs cannot take
 template <int RECON, bool DAG, bool EO, bool NC>
 __device__ __noinline__ void half_native(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                          int hh, C<double> (&acc)[9]) {
@@ -935,20 +950,21 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
         if (!native) {
             FxAcc acc;
 #pragma unroll
-            for (int k = 0; k < 18; ++k) acc.v[k] = 0;
+            for (int k = 0; k < 12; ++k) acc.v[k] = 0;
             acc.E = kFxMinExp;
             acc.bad = 0;
-            if (on) fx_hopping<RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
-            // bring both lanes of the site to one unit, then complete spin 3 - hh
+            if (on) fx_hopping<RECON, DAG, EO, NC, 1>(g, in, gauge, gdir_bytes, s, hh, acc);
+            // both lanes in one unit; the partner's spin 2 + hh' is this lane's 3 - hh
             const int Ep = __shfl_xor_sync(0xffffffffu, acc.E, 16);
-            const int E = max(acc.E, Ep), sh = min(E - acc.E, 63), e = E - 1022 - kFxSpinorBits;
+            if (Ep > acc.E) fx_raise(acc, Ep);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                const long long o = __shfl_xor_sync(0xffffffffu, acc.v[12 + k] >> sh, 16);
-                const long long up = acc.v[k] >> sh, dn = (acc.v[6 + k] >> sh) + o;
-                const double a = fx_value(up, e), b = fx_value(dn, e);
-                if (k & 1) { own[k / 2].im = a; own[3 + k / 2].im = b; }
-                else { own[k / 2].re = a; own[3 + k / 2].re = b; }
+            for (int k = 6; k < 12; ++k) acc.v[k] = __shfl_xor_sync(0xffffffffu, acc.v[k], 16);
+            if (on) fx_hopping<RECON, DAG, EO, NC, 0>(g, in, gauge, gdir_bytes, s, hh, acc);
+            const int e = acc.E - 1022 - kFxAccBits;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                own[k] = C<R>{fx_value(acc.v[2 * k], e), fx_value(acc.v[2 * k + 1], e)};
+                own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
             }
             native = acc.bad;
         }
@@ -1041,9 +1057,9 @@ __device__ __forceinline__ void store_part(const Pt &pt, void *base, int Vs, int
 
 // Register budget: the FP32 and FP16 kernels are memory-bound and want many
 // resident warps, so they are held to 3 blocks of 256 threads per SM (at most 85
-// registers); the fixed-point FP64 hops wait on integer results and loads and are held to
-// 128 (the compiler's 144: 1013 against 880-903 us at 32^3 x 64; 112 registers 889, 96 with
-// more spills 907); DF32 is arithmetic-bound and keeps the compiler's choice.
+// registers); the FP64 hops wait on results of the integer and FP64 pipes and are held to 128
+// (32^3 x 64: 811-850 us; 112 registers 841-848, 96 827-833 and slower on small lattices);
+// DF32 is arithmetic-bound and keeps the compiler's choice.
 template <int P> constexpr int dslash_min_blocks() { return (P == F32 || P == F16) ? 3 : P == F64 ? 2 : 0; }
 
 // Site tile (tile_x, in [0, gridDim.x)) and right-hand-side group (tile_y, in

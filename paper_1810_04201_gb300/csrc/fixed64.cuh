@@ -1,48 +1,50 @@
-// FP64 links and half spinors as 58-bit fixed-point numbers, and their products on the
-// integer multiply-add pipe (sm_103a).
+// FP64 links and half spinors as integer and float limbs, and their products off the FP64 pipe
+// (sm_103a).
 //
 // GB300 issues 2 FP64 operations per SM and clock (conversions between doubles and integers
 // included), so the 840 operations a site takes bound the FP64 operator at 420 clocks per site
-// and SM, ten times its HBM time.  The integer pipes are wider: a 32 x 32-bit multiply-add onto
-// a 64-bit sum costs four cycles of a scheduler where an FP64 multiply-add costs 64.  A link
-// entry is at most one in modulus, so it is kept as u = (H 2^29 + L) 2^-58 with
-// -2^28 <= L < 2^28, and a half spinor as (H 2^29 + L) 2^-57 in units of the power of two above
-// the largest component that the lane has met.  A real product is then three integer
-// multiply-adds,
-//   H H' 2^58 + (H L' + L H') 2^29   (L L' is dropped: about a unit of 2^-57 per hop),
-// a complex one nine (three real products), and the sums are exact: one rounding per link
-// product and one when the sum of the eight hops becomes a double.  FP64 arithmetic rounds each
-// partial sum to 2^-53 of itself, so the result is as close to the exact operator as before:
-// 1.5e-16 relative on Haar links and Gaussian spinors for both (64-bit reference summed in
-// another order; the rounding of the result itself).
-// Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 903 us, 16^4 107 -> 36 us; with
-// recon-12 links 5066 -> 1400 us.
+// and SM, ten times its HBM time.  A 32 x 32-bit multiply-add onto a 64-bit sum costs four cycles
+// of a scheduler, an FP32 one one, an FP64 one 64.  So a link entry, at most one in modulus, is
+// kept as u = H 2^-30 + L 2^-62, H an integer and L a float, and a half spinor likewise in units
+// of the power of two above the largest component that the lane has met.  A real product is
+//   H H' 2^-60   exact, summed in 64-bit integers, and
+//   (H L' + L H') 2^-92   in FP32,
+// and the sum of the eight hops, an integer in 2^-57 units, becomes a double with one rounding.
+// FP64 arithmetic rounds each partial sum to 2^-53 of itself; the FP32 products are off by 2^-24
+// of 2^-30: the result is closer to the exact operator than with FP64 arithmetic (relative error
+// against 128-bit arithmetic, Haar links, Gaussian spinors: kappa 0.12 8.2e-17 -> 6.2e-17, kappa 1
+// 1.57e-16 -> 1.01e-16, recon-12 at kappa 0.12 1.06e-16 -> 9.1e-17).
+// Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 811-850 us (128- and 64-thread blocks),
+// 16^4 107 -> 34.5 us; with recon-12 links 5066 -> 1083 us.  (Three integer products of 29-bit
+// limbs per real product, the first form: 882-888, 36.5 and 1400 us.)  What bounds it now is the
+// latency of its integer and FP64 results with 16 warps per SM: the integer and multiply-add pipes
+// are busy 41 and 37 % of the cycles, FP64 37 %, DRAM 20 %.
 //
-// Bounds.  Spinor components (a sum of two doubles) have |H| < 2^29, |L| < 2^30; links
-// |H| <= 2^29 (1 + 2^-11), |L| <= 2^28 and rows and columns of norm at most 1 + 2^-10.  The
-// largest sum, the middle one of (ur + ui)(x + y), is below
-// sqrt(2) 2^29 sqrt(3) 2^31 + 3 2^29 2^30 < 2^62.2; a hop is below sqrt(3) 2^58.6 < 2^59.4
-// and eight hops below 2^62.4.
+// Bounds.  A spinor component is a sum of two doubles, each below (1 - 2^-21) units, so H fits 32
+// bits; |L| <= 2^31; links |H| <= 2^30 (1 + 2^-11) with rows and columns of norm at most
+// 1 + 2^-10.  By Cauchy and Schwarz a sum of six products H H' is below sqrt(6) 2^61 (1 + 2^-10)
+// < 2^62.3, the small ones, in units of the sums, below 2^30, one hop below sqrt(6) 2^58 and
+// eight hops below 2^62.3.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace wd {
 
-constexpr int kFxBits = 29;                      // bits of a low limb
-constexpr double kFxLinkScale = 0x1p58;          // a link entry of one
-constexpr int kFxSpinorBits = 57;                // a spinor component of one unit
+constexpr double kFxLinkScale = 0x1p30;          // H of a link entry of one
+constexpr int kFxAccBits = 57, kFxAccShift = 3;  // products come in units 2^-60, sums in 2^-57
+constexpr long long kFxHalfAcc = 1ll << (kFxAccShift - 1);
+constexpr float kFxSmallToAcc = 0x1p-35f;        // small products come in units 2^-92
 // Exponents (biased) of the units this arithmetic takes: below, a scaled result could be
 // subnormal; above, the sum of eight hops could overflow.  Other fields go through FP64.
 constexpr int kFxMinExp = 128, kFxMaxExp = 2030;
 
-// link entry -> limbs
+// link entry -> (H, bits of the float L): u = H 2^-30 + L 2^-62
 __device__ __forceinline__ int2 fx_link(double u) {
-    const long long f = __double2ll_rn(u * kFxLinkScale);
-    const int h = (int)((f + (1ll << (kFxBits - 1))) >> kFxBits);
-    return make_int2(h, (int)(f - ((long long)h << kFxBits)));
+    const int h = __double2int_rn(u * kFxLinkScale);
+    return make_int2(h, __float_as_int((float)(fma((double)h, -0x1p-30, u) * 0x1p62)));
 }
 __device__ __forceinline__ double fx_link_value(int h, int l) {
-    return fma((double)h, 0x1p-29, (double)l * 0x1p-58);
+    return fma((double)h, 0x1p-30, (double)__int_as_float(l) * 0x1p-62);
 }
 
 // the larger of m and the |hi words| of two doubles, as float bits; NaN for words from
@@ -54,38 +56,63 @@ __device__ __forceinline__ float fx_max(float m, double a, double b) {
     return r;
 }
 
-// |d| in units 2^(E - 1022 - 57), E >= the exponent of d: high limb (28 bits) and low limb
-// (29 bits), truncated; c = ((E + 4) << 21) | 0x1fffff
-__device__ __forceinline__ void fx_limbs(double d, unsigned c, int &h, int &l) {
+// |d| in units 2^(E - 1022 - 62), truncated; E + 1 above the exponent of d;
+// c = ((E + 2) << 21) | 0x1fffff
+__device__ __forceinline__ unsigned long long fx_fixed(double d, unsigned c) {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
-    const unsigned n = (c - 2u * hi) >> 21;  // E + 4 - (exponent of d); the sign drops out
+    const unsigned n = (c - 2u * hi) >> 21;  // E + 2 - (exponent of d); the sign drops out
     const unsigned a = __funnelshift_l(lo, hi, 11) | 0x80000000u, b = lo << 11;
-    unsigned gl, gh;
-    asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%2, %3};\n\tshr.u64 t, t, %4;\n\tmov.b64 {%0, %1}, t;\n\t}"
-        : "=r"(gl), "=r"(gh) : "r"(b), "r"(a), "r"(n));
-    h = (int)gh;
-    l = (int)(gl >> 3);
+    unsigned long long t;
+    asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tshr.u64 %0, t, %3;\n\t}" : "=l"(t) : "r"(b), "r"(a), "r"(n));
+    return t;
 }
-
-// limbs of (-1)^ma |a| + (-1)^mb |b| with ma, mb = 0 or -1, times the signs of a and b
-__device__ __forceinline__ void fx_sum(double a, int ma, double b, int mb, unsigned c, int &h, int &l) {
-    int ha, la, hb, lb;
-    fx_limbs(a, c, ha, la);
-    fx_limbs(b, c, hb, lb);
+// s 2^-62 units as H 2^-30 + L 2^-62, |L| <= 2^31
+__device__ __forceinline__ void fx_split(long long s, int &h, float &l) {
+    const int lo = (int)s;
+    h = (int)(s >> 32) + (int)((unsigned)lo >> 31);
+    l = (float)lo;
+}
+// limbs of (-1)^m d (m = 0 or -1)
+__device__ __forceinline__ void fx_limbs(double d, int m, unsigned c, int &h, float &l) {
+    m ^= __double2hiint(d) >> 31;
+    fx_split((long long)(fx_fixed(d, c) ^ (unsigned long long)(long long)m) - m, h, l);
+}
+// limbs of (-1)^ma a + (-1)^mb b
+__device__ __forceinline__ void fx_sum(double a, int ma, double b, int mb, unsigned c, int &h, float &l) {
     ma ^= __double2hiint(a) >> 31;
     mb ^= __double2hiint(b) >> 31;
-    const int k = -ma - mb;
-    h = (ha ^ ma) + (hb ^ mb) + k;
-    l = (la ^ ma) + (lb ^ mb) + k;
+    fx_split((long long)(fx_fixed(a, c) ^ (unsigned long long)(long long)ma) +
+             (long long)(fx_fixed(b, c) ^ (unsigned long long)(long long)mb) - (ma + mb), h, l);
 }
 
 __device__ __forceinline__ long long fx_mac(int a, int b, long long s) { return (long long)a * b + s; }
 
-// s x 2^(e), e = (exponent of the unit) - 1022 - 57: the double nearest to the integer s,
-// moved by the exponent (kFxMinExp..kFxMaxExp keep it normal)
-__device__ __forceinline__ double fx_value(long long s, int e) {
-    const double d = (double)s;
-    return s == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+// (hr, hi, fr, fi) += u z (ADJ: conj(u) z) for a link entry u and z = x + iy with limbs
+// (x, xf = float(x), xl) and likewise y; mre, mim: the factors of u's imaginary limb in the
+// real and the imaginary part (ADJ ? y : -y, ADJ ? -x : x).  hr, hi: exact products of the high
+// limbs; fr, fi: the cross products in FP32, in units 2^-32 of those.
+template <bool ADJ>
+__device__ __forceinline__ void fx_cmac(int4 u, int x, int mre, int y, int mim, float xf, float yf, float xl, float yl,
+                                        long long &hr, long long &hi, float &fr, float &fi) {
+    const float rf = (float)u.x, rl = __int_as_float(u.y), jf = ADJ ? -(float)u.z : (float)u.z,
+                jl = ADJ ? -__int_as_float(u.w) : __int_as_float(u.w);
+    hr = fx_mac(u.z, mre, fx_mac(u.x, x, hr));
+    hi = fx_mac(u.z, mim, fx_mac(u.x, y, hi));
+    fr = fmaf(-jl, yf, fmaf(-jf, yl, fmaf(rl, xf, fmaf(rf, xl, fr))));
+    fi = fmaf(jl, xf, fmaf(jf, xl, fmaf(rl, yf, fmaf(rf, yl, fi))));
+}
+
+// The link entry of the value h 2^-60 + f 2^-92
+__device__ __forceinline__ int2 fx_link_of(long long h, float f) {
+    const int q = (int)((h + (1ll << 29)) >> 30);
+    const int r = (int)(h - ((long long)q << 30));
+    return make_int2(q, __float_as_int(fmaf((float)r, 4.f, f * 0x1p-30f)));
+}
+
+// v 2^e as a double, rounded once; e = (exponent of the unit) - 1022 - kFxAccBits
+__device__ __forceinline__ double fx_value(long long v, int e) {
+    const double d = (double)v;
+    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
 }
 
 }  // namespace wd

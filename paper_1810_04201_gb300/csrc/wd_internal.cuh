@@ -3,7 +3,7 @@
 // Field layouts are described in include/wd.h.  Gauge layouts (per direction mu,
 // blocks of Vs sites, complex entries row-major A*3+B):
 //   F64 recon-18: 9 arrays of Vs int4               recon-12: 6 arrays (rows 0, 1)
-//     (re.H, re.L, im.H, im.L): 58-bit fixed point, see fixed64.cuh; links that are not
+//     (re.H, re.L, im.H, im.L): integer and float limbs, see fixed64.cuh; links that are not
 //     unitary (Geom::links_fx = 0) are kept as double2 instead
 //   F32 recon-18: 4 arrays of Vs float4 (entries 0-7) + 1 array of Vs float2 (entry 8)
 //   F32 recon-12: 3 arrays of Vs float4
@@ -99,7 +99,7 @@ struct Geom {
     unsigned *dbg;   // debug builds: the context's word for the first out-of-range index
     int split_t;     // 1: one sub-lattice of a lattice split along t; the t hops that leave it
                      // (from the first slice backward, from the last slice forward) are omitted
-    int links_fx;    // FP64 links of recon 18 and 12 are fixed-point limbs (0: doubles)
+    int links_fx;    // FP64 links of recon 18 and 12 are limbs (fixed64.cuh) (0: doubles)
 };
 
 // coordinates of site n of the full lattice
@@ -319,7 +319,7 @@ template <int P, int RECON> struct LinkIO;
 
 template <int RECON> struct LinkIO<F64, RECON> {
     using R = double;
-    // fx: the entries are fixed-point limbs (recon 18 and 12)
+    // fx: the entries are limbs (recon 18 and 12)
     static __device__ __forceinline__ void load(const void *dir_base, int Vs, int s, C<R> (&u)[9], bool fx) {
         const double2 *p = reinterpret_cast<const double2 *>(dir_base) + s;
         if constexpr (RECON == 8) {

@@ -1,4 +1,4 @@
-"""The FP64 operator's fixed-point hops at the edges of their range: spinors of very different
+"""The FP64 operator's hops on integer and float limbs at the edges of their range: spinors of very different
 magnitude next to one another, zero and tiny and huge ones, and links that are not unitary
 (which go through FP64 arithmetic), against the oracle."""
 import numpy as np
@@ -37,8 +37,9 @@ def neighbourhood_max(psi, dims):
 @pytest.mark.parametrize("decades", [0, 3, 20, 120])
 def test_magnitudes_that_differ_between_neighbours(recon, decades):
     """Sites scaled by 10^(+-decades): each site's error is bounded by its own neighbourhood's
-    largest component (the unit of a lane is at most twice that, its resolution 2^-57: eight
-    hops of at most 16 units at |kappa| < 1, and the FP64 rounding of the oracle, stay below 2e-15)."""
+    largest component M.  The unit is at most 2 M; the FP32 products are off by 2^-24 of 12 terms
+    of 2^-30 units a hop, eight hops at kappa = 0.12 by 2e-15 / 5 M; the FP64 rounding of the oracle
+    and of the result stays below the rest of 2e-15 M."""
     U = gen.haar_links(DIMS, seed=3)
     psi = gen.gaussian_source(DIMS, seed=4)
     s = 10.0 ** (decades * (2.0 * gen.uniform(5, gen.STREAM_MISC, 0, psi.shape[0]) - 1.0))
