@@ -611,3 +611,27 @@ def test_fixed_rhs_tile_in_solver(wd):
         xs[rt] = lat.unpack(fx, nrhs=5, squeeze=False)
     for rt in (1, 2, 5):
         assert oracle.rel_err(xs[rt], xs[0]) < 1e-9
+
+
+@pytest.mark.parametrize("inner", [1, 2, 3])
+@pytest.mark.parametrize("nrhs,tol,max_iter", [(1, 1e-10, 1000), (3, 1e-8, 1000), (2, 1e-10, 5)])
+def test_even_odd_reports_the_residuals_of_what_it_returns(wd, inner, nrhs, tol, max_iter):
+    """The residuals that an even-odd reliable update reports for the whole lattice against the
+    oracle's of the returned solution (equal but for the rounding of b - D x, 1e-16 |b|)."""
+    dims, kappa = (4, 4, 6, 8), 0.12
+    U = gen.haar_links(dims, seed=11)
+    B = gen.gaussian_source(dims, seed=12, nrhs=nrhs)
+    lat = wd.Lattice(dims)
+    lat.set_gauge(U)
+    fx = lat.new_field(nrhs=nrhs)
+    res, _ = lat.cg(kappa, lat.pack(B), fx, tol=tol, max_iter=max_iter, inner=inner, nrhs=nrhs, precondition=1,
+                    raise_on_fail=False)
+    X = lat.unpack(fx, 0, nrhs, squeeze=False)
+    for k in range(nrhs):
+        r = B[k] - oracle.apply_D(U, X[k], kappa, dims)
+        n = oracle.apply_Ddag(U, r, kappa, dims)
+        want_b = np.linalg.norm(r) / np.linalg.norm(B[k])
+        want_n = np.linalg.norm(n) / np.linalg.norm(oracle.apply_Ddag(U, B[k], kappa, dims))
+        assert abs(res[k]["true_rel_resid_b"] - want_b) < 1e-4 * want_b + 4e-16
+        assert abs(res[k]["true_rel_resid"] - want_n) < 1e-4 * want_n + 4e-16
+        assert (res[k]["status"] == 0) == (want_n <= tol)
