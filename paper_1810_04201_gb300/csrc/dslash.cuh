@@ -1055,12 +1055,17 @@ __device__ __forceinline__ void store_part(const Pt &pt, void *base, int Vs, int
     }
 }
 
-// Register budget: the FP32 and FP16 kernels are memory-bound and want many
-// resident warps, so they are held to 3 blocks of 256 threads per SM (at most 85
-// registers); the FP64 hops wait on results of the integer and FP64 pipes and are held to 128
+// Register budget, as blocks of 256 threads per SM.  FP16 and FP32 with compressed links are held
+// to three (at most 85 registers) for the resident warps: 32^3 x 64 us, three / two blocks: FP16
+// 127 / 161, FP16 recon-12 129 / 139, FP32 recon-12 162 / 165.  FP32 with whole links to two
+// (128 registers), which keep the loads of two hops in flight: 194 -> 188 us at 32^3 x 64,
+// 10.3 -> 8.3 at 16^4 (four blocks: 64 registers, spills, 305 us; one: 215 registers, 235 us).
+// The FP64 hops wait on results of the integer and FP64 pipes and are held to 128 registers
 // (32^3 x 64: 811-850 us; 112 registers 841-848, 96 827-833 and slower on small lattices);
 // DF32 is arithmetic-bound and keeps the compiler's choice.
-template <int P> constexpr int dslash_min_blocks() { return (P == F32 || P == F16) ? 3 : P == F64 ? 2 : 0; }
+template <int P, int RECON> constexpr int dslash_min_blocks() {
+    return P == F64 || (P == F32 && RECON == 18) ? 2 : P == F32 || P == F16 ? 3 : 0;
+}
 
 // Site tile (tile_x, in [0, gridDim.x)) and right-hand-side group (tile_y, in
 // [0, gridDim.y)) of this block.  Blocks start in linear order (x fastest); numbering
@@ -1082,7 +1087,7 @@ __device__ __forceinline__ int tile_y() {
 // lane's two spins); Ep::finish runs once per thread after the loop (block and grid
 // reductions, solver scalars).
 template <int P, int RECON, bool DAG, class Ep, bool EO = false>
-__global__ void __launch_bounds__(256, dslash_min_blocks<P>()) dslash_kernel(DslashArgs a) {
+__global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_kernel(DslashArgs a) {
     using R = typename Real<P>::T;
     if (a.run_flag && *a.run_flag == 0) return;
     const int r = tile_y() * blockDim.y + threadIdx.y;
