@@ -89,20 +89,20 @@ static inline int num_sms() {
 }
 
 // Grid for a reducing Dslash (one partial per block and row; the partial buffers hold
-// kMaxPartialBlocks per row).  Up to that many site tiles get one block each and the
-// hardware scheduler balances them across the SMs to the end of the launch; larger
-// lattices get the blocks that are resident at once, each walking many tiles.
+// kMaxPartialBlocks per row): the blocks that are resident at once, each walking many site tiles,
+// so that the block reduction, the fence and the ticket are paid once per block.  One block per
+// tile, left to the hardware scheduler, is slower wherever there are more tiles than that (solves,
+// ms: 24^4 FP32 8.11 against 6.88, FP16 6.62 / 5.69; 20^3 x 40 FP32 with 12 rows 70.4 / 62.2;
+// 16^3 x 32 FP64 9.41 / 8.44), and so are half and twice as many blocks (24^4 FP32 8.62, 7.51).
 constexpr int kMaxPartialBlocks = 8192;
 template <int P, class K>
 static dim3 reduce_grid(K kernel, const Geom &g, DslashTiles t, int nrhs) {
-    const dim3 rows(1, (nrhs + t.rhs_tile - 1) / t.rhs_tile);
-    const int need = site_blocks<P>(g.V, t.site_tile);
-    if (need <= kMaxPartialBlocks) return dim3(need, rows.y);
+    const int need = site_blocks<P>(g.V, t.site_tile), rows = (nrhs + t.rhs_tile - 1) / t.rhs_tile;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, t.site_tile * t.rhs_tile, 0);
     if (per_sm < 1) per_sm = 1;
-    const int cap = per_sm * num_sms();
-    return dim3(cap < kMaxPartialBlocks ? cap : kMaxPartialBlocks, rows.y);
+    const int cap = per_sm * num_sms() < kMaxPartialBlocks ? per_sm * num_sms() : kMaxPartialBlocks;
+    return dim3(need < cap ? need : cap, rows);
 }
 
 // Even-odd preconditioning: the solver works on the even half of the lattice
