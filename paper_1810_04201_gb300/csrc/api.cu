@@ -200,15 +200,24 @@ void graph_clear(wd_ctx *c) {
 
 // Where no autotuner or wd_set_tiles chose a shape, the fused kernels take up to four right-hand
 // sides per block (12 rows of FP32 at 24^3 x 48: 128.9 ms a solve against 129.8 with one and
-// 130.8 with two per block; the plain operators differ, see tiles_for).
+// 130.8 with two per block; the plain operators differ, see tiles_for).  FP32 rows go in pairs on
+// one thread from 2^17 site-rows on with four rows (24^3 x 48: 41.3 -> 39.6 ms) and, even-odd, with
+// more (20^3 x 40, 12 rows 37.9 -> 36.3); two rows gain nothing (21.2 / 21.7 ms), and 12 rows on the
+// whole lattice lose (126 / 134 ms).
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
     if (it != c->cg_tiles.end()) return it->second;
     it = c->tiles.find(p * 64 + nrhs);
-    if (it != c->tiles.end()) return it->second;
     DslashTiles t;
+    if (it != c->tiles.end()) {
+        t = it->second;
+        t.rhs_per_thread = 1;  // chosen for the plain operators
+        return t;
+    }
     t.site_tile = 64;
     t.rhs_tile = nrhs < 4 ? nrhs : 4;
+    const long long work = (long long)c->g.V * nrhs / (eo ? 2 : 1);
+    if (p == F32 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) && work >= (1 << 17)) t.rhs_per_thread = 2;
     return t;
 }
 

@@ -185,8 +185,8 @@ wd_status wd_cg_solve(wd_ctx *c, double kappa, const void *b, void *x, const wd_
         }
     }
     char key[256];
-    snprintf(key, sizeof key, "cg|%d|%d|%d,%d|%a|%d,%d|%d,%d|%d|%d|%d", (int)inner, nrhs, r64, rin, kappa,
-             pl.t64.site_tile, pl.t64.rhs_tile, pl.tin.site_tile, pl.tin.rhs_tile, pl.ne, pl.eo,
+    snprintf(key, sizeof key, "cg|%d|%d|%d,%d|%a|%d,%d|%d,%d,%d|%d|%d|%d", (int)inner, nrhs, r64, rin, kappa,
+             pl.t64.site_tile, pl.t64.rhs_tile, pl.tin.site_tile, pl.tin.rhs_tile, pl.tin.rhs_per_thread, pl.ne, pl.eo,
              corr ? 1 + f.c32_inner : 0);
     const char *loop_env = getenv("WD_CG_LOOP");
     const bool host_loop = loop_env && std::strcmp(loop_env, "host") == 0;

@@ -34,17 +34,20 @@ template <int N> __device__ __forceinline__ double norm2_of(const C<float> (&v)[
     return (double)n;
 }
 
-// Block + grid reduction of NV doubles per row; `fin(row, tot)` runs once per
-// enabled row, in thread (0, 0) of the last block, rows in order.
-template <int NV, class F>
-__device__ __forceinline__ bool reduce_finish(const DslashArgs &a, double (&v)[NV], F &&fin) {
+// Block + grid reduction of the NV doubles of each of the thread's K rows r, r + 1, ...;
+// `fin(row, tot)` runs once per enabled row, in thread (0, 0) of the last block, rows in order.
+template <int NV, int K, class St, class F>
+__device__ __forceinline__ bool reduce_finish(const DslashArgs &a, int r, St (&st)[K], F &&fin) {
     __shared__ double smem[WD_MAX_RHS * 8 * NV];
     __shared__ double tot[WD_MAX_RHS * NV];
-    block_reduce_rows<NV>(v, smem);
-    const int r = tile_y() * blockDim.y + threadIdx.y;
-    if (threadIdx.x == 0 && r < a.nrhs)
 #pragma unroll
-        for (int k = 0; k < NV; ++k) a.partial[((size_t)r * NV + k) * gridDim.x + tile_x()] = v[k];
+    for (int k = 0; k < K; ++k) {
+        if (k) __syncthreads();  // smem is read by the row before
+        block_reduce_rows<NV>(st[k].v, smem);
+        if (threadIdx.x == 0 && r + k < a.nrhs)
+#pragma unroll
+            for (int q = 0; q < NV; ++q) a.partial[((size_t)(r + k) * NV + q) * gridDim.x + tile_x()] = st[k].v[q];
+    }
     const bool last = last_block(a.counter);
     if (last) {
         sum_partials<NV>(a.partial, gridDim.x, a.nrhs, tot);
@@ -77,9 +80,9 @@ struct EpSetupDb {
         st.v[0] += norm2_of(p);
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, p);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<2>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<2>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             c.rhs2 = t[0];
             c.b2 = t[1];
@@ -110,9 +113,9 @@ struct EpSetupR {
         store_part<P>(pt, rhs_ptr<R>(a.a1, a.a1_stride, r), a.g.Vs, s, d);
         store_part<P>(pt, rhs_ptr<R>(a.a2, a.a2_stride, r), a.g.Vs, s, d);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             c.rho = t[0];
             c.rmax2 = t[0];
@@ -137,9 +140,9 @@ struct EpCG1 {
         st.v[0] += norm2_of(p);
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, p);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             c.pAp = t[0];
             if (!is_fin(t[0])) { c.status = WD_ERR_NONFINITE; c.active = 0; c.alpha = 0.0; }
@@ -172,9 +175,9 @@ struct EpCG2 {
         for (int c = 0; c < Pt::N; ++c) v[c] = C<R>{v[c].re + alpha * q[c].re, v[c].im + alpha * q[c].im};
         store_part<P>(pt, xr, a.g.Vs, s, v);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             const double rn = t[0];
             c.iter += 1;
@@ -215,11 +218,11 @@ struct EpCG2Mixed {
             xs[c] = C<float>{xs[c].re + float(alpha * q[c].re), xs[c].im + float(alpha * q[c].im)};
         store_part<F32>(pt, xr, a.g.Vs, s, xs);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
         __shared__ int any;
         if (threadIdx.x == 0 && threadIdx.y == 0) any = 0;
-        const bool last = reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+        const bool last = reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             const double rn = t[0];
             c.iter += 1;
@@ -263,9 +266,9 @@ struct EpResid {
         st.v[0] += norm2_of(b);
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, b);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) { a.sc[row].true_b2 = t[0]; });
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].true_b2 = t[0]; });
     }
 };
 
@@ -281,9 +284,9 @@ struct EpHopNorm {
         st.v[0] += norm2_of(acc);
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, acc);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) { a.sc[row].odd2 = t[0]; });
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].odd2 = t[0]; });
     }
 };
 
@@ -304,9 +307,9 @@ struct EpReliable {
         st.v[0] += norm2_of(d);
         store_part<P>(pt, rhs_ptr<R>(a.a1, a.a1_stride, r), a.g.Vs, s, d);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             const double rt = t[0];
             c.reliable += 1;
@@ -353,9 +356,9 @@ struct EpCorrect {
         st.v[0] += norm2_of(d);
         store_part<SP>(pt, rhs_ptr<float>(a.a1, a.a1_stride, r), a.g.Vs, s, d);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) {
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) {
             Scalars &c = a.sc[row];
             const double rt = t[0];
             c.corrections += 1;
@@ -383,9 +386,9 @@ struct EpTrue1 {
         for (int c = 0; c < Pt::N; ++c) b[c] = csub(b[c], p[c]);
         st.v[0] += norm2_of(b);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) { a.sc[row].true_b2 = t[0]; });
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].true_b2 = t[0]; });
     }
 };
 
@@ -403,9 +406,9 @@ struct EpTrue2 {
         for (int c = 0; c < Pt::N; ++c) d[c] = csub(d[c], q[c]);
         st.v[0] += norm2_of(d);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int, bool, State &st) {
-        reduce_finish<1>(a, st.v, [&](int row, const double *t) { a.sc[row].true_n2 = t[0]; });
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
+        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].true_n2 = t[0]; });
     }
 };
 

@@ -15,6 +15,7 @@
 //   D^dag: the signs swap (gamma5 D gamma5 = D^dag, section 2.2).
 //   Antiperiodic time boundary: the hop across t = T-1 <-> 0 is multiplied by -1.
 #pragma once
+#include <type_traits>
 #include "wd_internal.cuh"
 
 namespace wd {
@@ -1097,7 +1098,7 @@ __global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_ker
     // the field the xpay epilogues add: the hopping input unless another is given
     const void *xin = a.xsrc ? rhs_ptr<R>(a.xsrc, a.xsrc_stride, rr) : in;
     const bool zin = a.in_nonzero && *a.in_nonzero == 0;
-    typename Ep::State st{};
+    typename Ep::State st[1]{};
     if constexpr (split_site<P>()) {
         // two lanes per site (blockDim.x a multiple of 32): lane l of warp w of the
         // block takes site 16 w + (l mod 16), half l / 16
@@ -1111,7 +1112,7 @@ __global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_ker
             C<R> own[6];
             // all 32 lanes: row and s0 are the same for them
             hopping_own<P, RECON, DAG, EO>(a.g, in, a.gauge, a.gauge_dir, s, hh, on && !zin, own);
-            if (on) Ep::template site<P>(a, s, r, xin, own, st, pt);
+            if (on) Ep::template site<P>(a, s, r, xin, own, st[0], pt);
         }
     } else {
         const SiteAll pt{};
@@ -1124,11 +1125,11 @@ __global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_ker
                     for (int k = 0; k < 12; ++k) acc[k] = C<R>{R(0), R(0)};
                 else if constexpr (EO) hopping_eo<P, RECON, DAG>(a.g, in, a.gauge, a.gauge_dir, s, acc);
                 else hopping<P, RECON, DAG>(a.g, in, a.gauge, a.gauge_dir, s, acc);
-                Ep::template site<P>(a, s, r, xin, acc, st, pt);
+                Ep::template site<P>(a, s, r, xin, acc, st[0], pt);
             }
         }
     }
-    Ep::template finish<P>(a, r, row, st);
+    Ep::template finish<P>(a, r, st);
 }
 
 // ---------------------------------------------------------------- epilogues
@@ -1145,8 +1146,8 @@ struct EpXpay {
         for (int c = 0; c < Pt::N; ++c) p[c] = C<R>{p[c].re - k * acc[c].re, p[c].im - k * acc[c].im};
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, p);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &, int, bool, State &) {}
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &, int, State (&)[K]) {}
 };
 
 // out = -kappa * hop (no added field); kappa = -1 gives the bare hopping term
@@ -1160,8 +1161,8 @@ struct EpHop {
         for (int c = 0; c < Pt::N; ++c) acc[c] = C<R>{k * acc[c].re, k * acc[c].im};
         store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, acc);
     }
-    template <int P>
-    static __device__ __forceinline__ void finish(const DslashArgs &, int, bool, State &) {}
+    template <int P, int K>
+    static __device__ __forceinline__ void finish(const DslashArgs &, int, State (&)[K]) {}
 };
 
 template <class R, int N> __device__ __forceinline__ double norm2_of(const C<R> (&v)[N]) {
@@ -1172,41 +1173,38 @@ template <class R, int N> __device__ __forceinline__ double norm2_of(const C<R> 
 }
 
 // ---------------------------------------------------------------- K right-hand sides per thread
-// The plain FP32 operator with each thread applying its site's links to K right-hand sides:
-// a link is loaded once and multiplies K projected half spinors, so per site and right-hand
-// side the loads of links (288 bytes, 40 instructions) fall K-fold; the spinor loads are the
-// same.  Rows past nrhs (a partial last group) read a valid row and store nothing.
+// FP32 with each thread applying its site's links to K right-hand sides: a link is loaded once
+// and multiplies K projected half spinors, so per site and right-hand side the loads of links
+// (288 bytes, 40 instructions) fall K-fold; the spinor loads are the same.  Rows past nrhs (a
+// partial last group) and rows that the mask leaves out read a valid row and store nothing.
+// Forward neighbour nf with link gf[kf], backward neighbour nb with link gb[nb].
 template <int RECON, bool DAG, int MU, int K>
-__device__ __forceinline__ void hop_dir_k(const DslashArgs &a, const char *gdir, const int (&row)[K], int s, int c,
+__device__ __forceinline__ void hop_dir_k(const DslashArgs &a, const char *gf, int kf, int nf, bool flip_f,
+                                          const char *gb, int nb, bool flip_b, const int (&row)[K],
                                           C<float> (&acc)[K][12]) {
     constexpr int SF = DAG ? +1 : -1;
     const Geom &g = a.g;
-    const int L = g.L[MU], st = g.stride[MU];
     {
-        const int sf = WD_IDX(g, (c == L - 1) ? s - (L - 1) * st : s + st, g.V, 1);
         C<float> u[9];
-        LinkIO<F32, RECON>::load(gdir, g.Vs, s, u);
-        const bool flip = MU == 3 && g.antiperiodic && c == L - 1;
+        LinkIO<F32, RECON>::load(gf, g.Vs, kf, u);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             C<float> p[12], h[6], w[6];
-            SpinorIO<F32>::load(rhs_ptr<float>(a.in, a.in_stride, row[k]), g.Vs, sf, p);
+            SpinorIO<F32>::load(rhs_ptr<float>(a.in, a.in_stride, row[k]), g.Vs, nf, p);
             project<MU, SF>(p, h);
-            su3_mult<false>(u, h, w, flip);
+            su3_mult<false>(u, h, w, flip_f);
             accumulate<MU, SF>(acc[k], w);
         }
     }
     {
-        const int sb = WD_IDX(g, (c == 0) ? s + (L - 1) * st : s - st, g.V, 2);
         C<float> u[9];
-        LinkIO<F32, RECON>::load(gdir, g.Vs, sb, u);
-        const bool flip = MU == 3 && g.antiperiodic && c == 0;
+        LinkIO<F32, RECON>::load(gb, g.Vs, nb, u);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             C<float> p[12], h[6], w[6];
-            SpinorIO<F32>::load(rhs_ptr<float>(a.in, a.in_stride, row[k]), g.Vs, sb, p);
+            SpinorIO<F32>::load(rhs_ptr<float>(a.in, a.in_stride, row[k]), g.Vs, nb, p);
             project<MU, -SF>(p, h);
-            su3_mult<true>(u, h, w, flip);
+            su3_mult<true>(u, h, w, flip_b);
             accumulate<MU, -SF>(acc[k], w);
         }
     }
@@ -1214,40 +1212,65 @@ __device__ __forceinline__ void hop_dir_k(const DslashArgs &a, const char *gdir,
 
 // K = 2 is held to 128 registers (two blocks of 256 per SM; the compiler's choice is 152, and
 // the cap costs 32 bytes of spills): 4 % faster at 12 right-hand sides.  K = 3, 4 keep theirs.
-template <int RECON, bool DAG, int K>
+template <int RECON, bool DAG, int K, class Ep = EpXpay, bool EO = false>
 __global__ void __launch_bounds__(256, K == 2 ? 2 : 1) dslash_multi_kernel(DslashArgs a) {
+    if (a.run_flag && *a.run_flag == 0) return;
     const int r0 = (tile_y() * blockDim.y + threadIdx.y) * K;
-    if (r0 >= a.nrhs) return;  // no block-wide step follows
     int row[K];
+    bool on[K], any = false;
 #pragma unroll
-    for (int k = 0; k < K; ++k) row[k] = r0 + k < a.nrhs ? r0 + k : a.nrhs - 1;
-    const char *gb = reinterpret_cast<const char *>(a.gauge);
-    for (int s0 = tile_x() * blockDim.x; s0 < a.g.V; s0 += gridDim.x * blockDim.x) {
+    for (int k = 0; k < K; ++k) {
+        on[k] = r0 + k < a.nrhs && row_on(a.sc, a.mask, r0 + k);
+        any |= on[k];
+        row[k] = r0 + k < a.nrhs ? r0 + k : a.nrhs - 1;
+    }
+    const bool zin = a.in_nonzero && *a.in_nonzero == 0;
+    const Geom &g = a.g;
+    const char *gp = reinterpret_cast<const char *>(a.gauge), *gq = gp;
+    if constexpr (EO) {
+        gp += (size_t)(4 * g.eo_parity) * a.gauge_dir;
+        gq += (size_t)(4 * (1 - g.eo_parity)) * a.gauge_dir;
+    }
+    typename Ep::State st[K]{};
+    for (int s0 = tile_x() * blockDim.x; s0 < g.V; s0 += gridDim.x * blockDim.x) {
         const int s = s0 + threadIdx.x;
-        if (s >= a.g.V) continue;
-        int x, y, z, t;
-        site_xyzt(a.g, s, x, y, z, t);
+        if (s >= g.V || !any) continue;
         C<float> acc[K][12];
 #pragma unroll
         for (int k = 0; k < K; ++k)
 #pragma unroll
             for (int c = 0; c < 12; ++c) acc[k][c] = C<float>{0.f, 0.f};
-        hop_dir_k<RECON, DAG, 0, K>(a, gb, row, s, x, acc);
-        hop_dir_k<RECON, DAG, 1, K>(a, gb + a.gauge_dir, row, s, y, acc);
-        hop_dir_k<RECON, DAG, 2, K>(a, gb + 2 * a.gauge_dir, row, s, z, acc);
-        hop_dir_k<RECON, DAG, 3, K>(a, gb + 3 * a.gauge_dir, row, s, t, acc);
-        const float kap = (float)a.kappa;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if (r0 + k >= a.nrhs) break;
-            C<float> p[12];
-            SpinorIO<F32>::load(a.xsrc ? rhs_ptr<float>(a.xsrc, a.xsrc_stride, row[k]) : rhs_ptr<float>(a.in, a.in_stride, row[k]),
-                                a.g.Vs, s, p);
-#pragma unroll
-            for (int c = 0; c < 12; ++c) p[c] = C<float>{p[c].re - kap * acc[k][c].re, p[c].im - kap * acc[k][c].im};
-            SpinorIO<F32>::store(rhs_ptr<float>(a.out, a.out_stride, row[k]), a.g.Vs, s, p);
+        if (!zin) {
+            int xc[4], m = s;
+            if constexpr (EO) m = eo_full_index(g, s, xc[0], xc[1], xc[2], xc[3]);
+            else site_xyzt(g, s, xc[0], xc[1], xc[2], xc[3]);
+            auto dir = [&](auto muc) {
+                constexpr int MU = decltype(muc)::value;
+                const int L = g.L[MU], sd = g.stride[MU], c = xc[MU];
+                int nf = WD_IDX(g, (c == L - 1) ? m - (L - 1) * sd : m + sd, EO ? 2 * g.V : g.V, EO ? 3 : 1);
+                int nb = WD_IDX(g, (c == 0) ? m + (L - 1) * sd : m - sd, EO ? 2 * g.V : g.V, EO ? 4 : 2);
+                if (EO) {
+                    nf >>= 1;
+                    nb >>= 1;
+                }
+                hop_dir_k<RECON, DAG, MU, K>(a, gp + (size_t)MU * a.gauge_dir, s, nf,
+                                             MU == 3 && g.antiperiodic && c == L - 1, gq + (size_t)MU * a.gauge_dir, nb,
+                                             MU == 3 && g.antiperiodic && c == 0, row, acc);
+            };
+            dir(std::integral_constant<int, 0>{});
+            dir(std::integral_constant<int, 1>{});
+            dir(std::integral_constant<int, 2>{});
+            dir(std::integral_constant<int, 3>{});
         }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (on[k])
+                Ep::template site<F32>(a, s, r0 + k,
+                                       a.xsrc ? rhs_ptr<float>(a.xsrc, a.xsrc_stride, row[k])
+                                              : rhs_ptr<float>(a.in, a.in_stride, row[k]),
+                                       acc[k], st[k], SiteAll{});
     }
+    Ep::template finish<F32>(a, r0, st);
 }
 
 }  // namespace wd

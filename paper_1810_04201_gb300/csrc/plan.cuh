@@ -6,6 +6,7 @@
 #include <vector>
 #include "dslash.cuh"
 #include "blas.cuh"
+#include "cg_kernels.cuh"
 
 namespace wd {
 
@@ -96,10 +97,10 @@ static inline int num_sms() {
 // 16^3 x 32 FP64 9.41 / 8.44), and so are half and twice as many blocks (24^4 FP32 8.62, 7.51).
 constexpr int kMaxPartialBlocks = 8192;
 template <int P, class K>
-static dim3 reduce_grid(K kernel, const Geom &g, DslashTiles t, int nrhs) {
+static dim3 reduce_grid(K kernel, const Geom &g, DslashTiles t, int nrhs, int threads) {
     const int need = site_blocks<P>(g.V, t.site_tile), rows = (nrhs + t.rhs_tile - 1) / t.rhs_tile;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, t.site_tile * t.rhs_tile, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
     if (per_sm < 1) per_sm = 1;
     const int cap = per_sm * num_sms() < kMaxPartialBlocks ? per_sm * num_sms() : kMaxPartialBlocks;
     return dim3(need < cap ? need : cap, rows);
@@ -130,13 +131,24 @@ struct Fields {
     EoInfo eo;
 };
 
+// the kernels of the FP32 inner iteration, which also take two right-hand sides per thread
+template <class Ep> constexpr bool pairs_rows() {
+    return std::is_same_v<Ep, EpCG1> || std::is_same_v<Ep, EpCG2Mixed> || std::is_same_v<Ep, EpHop>;
+}
+
 template <int P, int RECON, bool DAG, class Ep, bool EO = false>
 static void add_dslash(GraphBuilder &gb, const DslashArgs &a, DslashTiles t, bool reduce) {
-    auto k = dslash_kernel<P, RECON, DAG, Ep, EO>;
-    dim3 block(t.site_tile, t.rhs_tile);
-    dim3 grid = reduce ? reduce_grid<P>(k, a.g, t, a.nrhs)
-                       : dim3(site_blocks<P>(a.g.V, t.site_tile), (a.nrhs + t.rhs_tile - 1) / t.rhs_tile);
-    gb.kernel(k, grid, block, a);
+    const int per = P == F32 && pairs_rows<Ep>() && t.rhs_per_thread == 2 && t.rhs_tile % 2 == 0 ? 2 : 1;
+    const dim3 block(t.site_tile, t.rhs_tile / per);
+    auto add = [&](auto k) {
+        dim3 grid = reduce ? reduce_grid<P>(k, a.g, t, a.nrhs, block.x * block.y)
+                           : dim3(site_blocks<P>(a.g.V, t.site_tile), (a.nrhs + t.rhs_tile - 1) / t.rhs_tile);
+        gb.kernel(k, grid, block, a);
+    };
+    if constexpr (P == F32 && pairs_rows<Ep>()) {
+        if (per == 2) return add(dslash_multi_kernel<RECON, DAG, 2, Ep, EO>);
+    }
+    add(dslash_kernel<P, RECON, DAG, Ep, EO>);
 }
 
 template <class K>

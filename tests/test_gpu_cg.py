@@ -635,3 +635,31 @@ def test_even_odd_reports_the_residuals_of_what_it_returns(wd, inner, nrhs, tol,
         assert abs(res[k]["true_rel_resid_b"] - want_b) < 1e-4 * want_b + 4e-16
         assert abs(res[k]["true_rel_resid"] - want_n) < 1e-4 * want_n + 4e-16
         assert (res[k]["status"] == 0) == (want_n <= tol)
+
+
+@pytest.mark.parametrize("nrhs,eo", [(4, 0), (4, 1), (6, 1), (12, 1)])
+def test_rows_in_pairs_match_single_rows(wd, nrhs, eo):
+    """From 2^17 site-rows on the FP32 iteration takes two right-hand sides per thread: the same
+    arithmetic, so the solutions agree with those of one row per thread but for the order of the sums
+    over sites, which moves alpha and beta by a few 1e-16 (FP32 rounding of the iterates: 1e-7 of a
+    residual that the FP64 updates then correct, so both meet 1e-10; 16 sites of tile keep one row)."""
+    dims, kappa = (16, 16, 16, 16 if eo == 0 or nrhs > 4 else 32), 0.12
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(7)
+    U = gen.haar_links((4, 4, 4, 4), seed=5)
+    V = int(np.prod(dims))
+    Ug = torch.from_numpy(U).cuda().reshape(4, 256, 9).repeat(1, V // 256, 1).reshape(4, V, 3, 3).contiguous()
+    B = torch.complex(torch.randn(nrhs, V, 4, 3, generator=g, device="cuda", dtype=torch.float64),
+                      torch.randn(nrhs, V, 4, 3, generator=g, device="cuda", dtype=torch.float64))
+    lat = wd.Lattice(dims)
+    lat.set_gauge(Ug)
+    fb = lat.pack(B)
+    out = []
+    for paired in (True, False):
+        if not paired:
+            lat.set_tiles(1, nrhs, 64, 2)
+        fx = lat.new_field(nrhs=nrhs)
+        res, st = lat.cg(kappa, fb, fx, tol=1e-10, inner=1, nrhs=nrhs, precondition=eo)
+        assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
+        out.append(fx.view(torch.float64).clone())
+    assert float((out[0] - out[1]).norm() / out[1].norm()) < 2e-9
