@@ -3,7 +3,7 @@
 // updates (section 2.3: a new U and eta per solve; section 2.2: CG on the normal
 // equations).
 //
-// Work list: every lattice is cut into tiles of kTile sites; the tiles of all
+// Work list: every lattice is cut into tiles of 128 or 256 sites; the tiles of all
 // lattices form one list that the resident blocks walk (block b takes tiles b,
 // b + grid, ...).  A CG step is a sequence of phases separated by grid barriers;
 // per-lattice reductions use one partial per tile and the block that finishes a
@@ -30,8 +30,14 @@ using namespace wd;
 
 namespace wd {
 
-constexpr int kTile = 128;
-constexpr int kHalfTile = kTile / 2;  // sites of one pass of the two-lane FP64 phases
+constexpr int kThreads = 128;
+constexpr int kBlocksPerSm = 5;
+// Sites of a tile: two per thread, so that its reduction (two block barriers, a fence and a
+// ticket) and the copy of its lattice's description are paid once for both, where that leaves every
+// resident block at least four tiles; else one (64 lattices of 1.86 M sites, ms: 128 sites 39.6, 256
+// 36.1, 512, with uneven blocks, 40.8).
+inline int tile_sites(long long sites) { return sites >= 4ll * 256 * kBlocksPerSm * num_sms() ? 256 : 128; }
+constexpr int kHalfTile = kThreads / 2;  // sites of one pass of the two-lane FP64 phases
 constexpr int kPart = 4;              // partial sums per tile
 // A reliable update that delta triggers waits up to this many iterations, while the
 // lattice's CG steps go on, so that the updates of many lattices share one update phase
@@ -55,6 +61,7 @@ struct BatchArgs {
     double *tpart;       // per tile partials (2 values)
     const int *tile_lat; // lattice of each tile
     int ntiles, nlat, max_iter;
+    int tile;            // sites per tile, a multiple of kThreads
     unsigned *bar_count, *bar_gen;
     int *flags;          // [0] error, [1] any reliable update pending, [2] iterations run, [3] never set
     int *lstate;         // per lattice: [0] start vector nonzero, [1] the last reliable update was the final check
@@ -147,18 +154,19 @@ __device__ __forceinline__ void walk_tiles(const BatchArgs &a, LatDesc &L, W &&w
     }
 }
 
-// one thread per site: `body(L, g, l, s, valid)`
-template <class W, class F>
-__device__ void for_tiles(const BatchArgs &a, W &&want, F &&body) {
+// one thread per site: `body(L, l, s)` for every site of the tile, then `end(L, g, l)`
+template <class W, class F, class E>
+__device__ void for_tiles(const BatchArgs &a, W &&want, F &&body, E &&end) {
     __shared__ LatDesc L;
     walk_tiles(a, L, want, [&](const LatDesc &D, int g, int l) {
-        const int s = (g - D.tile0) * kTile + threadIdx.x;
-        body(D, g, l, s, s < D.g.V);
+        const int s0 = (g - D.tile0) * a.tile + threadIdx.x;
+        for (int s = s0; s < s0 + a.tile && s < D.g.V; s += kThreads) body(D, l, s);
+        end(D, g, l);
     });
 }
 
 // The FP64 phases run two lanes per site like the FP64 Dslash kernel: lanes l and
-// l ^ 16 of a warp share a site (lane half hh), so a tile takes two passes of
+// l ^ 16 of a warp share a site (lane half hh), so a tile takes passes of
 // kHalfTile sites; `body(L, g, l, sl, hh)` gets the lane's site offset sl within a pass.
 template <class W, class F>
 __device__ void for_tiles_half(const BatchArgs &a, W &&want, F &&body) {
@@ -178,13 +186,14 @@ __device__ __noinline__ void hop64_half(const LatDesc &L, const void *in, int s,
     hopping_own<F64, RECON, DAG, false, false>(L.g, in, L.g64, L.gdir64, s, hh, on, own);
 }
 
-// Five blocks of 128 threads per SM (96 registers): the inner FP32 phases, which wait on
-// loads, gain more from the extra warps than the FP64 phases lose to spills (C5: 54.0 ms
-// at four blocks, 52.7 at five).
+// kBlocksPerSm blocks of 128 threads per SM (96 registers): the inner FP32 phases, which wait on
+// loads, gain more from the extra warps than the FP64 phases lose to spills (64 lattices of
+// 1.86 M sites: 42.1 ms at three blocks, 39.5 at four, 38.5 at five).
 template <int SP, int RECON, int RIN>
-__global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm) k_batched_cg(BatchArgs a) {
     using RS = typename Real<SP>::T;
     auto all = [](const Scalars &, int) { return 1; };
+    auto none = [](const LatDesc &, int, int) {};
     auto active = [](const Scalars &c, int) { return c.active; };
     auto updating = [](const Scalars &c, int) { return c.active && (c.do_update || c.pending); };
     auto x0_nonzero = [&](const Scalars &, int l) { return a.lstate[2 * l]; };
@@ -203,8 +212,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
     for_tiles_half(a, all, [&](const LatDesc &L, int g, int l, int sl, int hh) {
         const SiteHalf pt{hh};
         double v[3] = {0.0, 0.0, 0.0};
-        for (int h2 = 0; h2 < 2; ++h2) {
-            const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+        for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+            const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
             const bool on = s < L.g.V;
             C<double> acc[6], p[6];
             hop64_half<RECON, true>(L, L.b, s, hh, on, acc);
@@ -230,8 +239,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
     // S2: t = D x0
     for_tiles_half(a, x0_nonzero, [&](const LatDesc &L, int g, int, int sl, int hh) {
         const SiteHalf pt{hh};
-        for (int h2 = 0; h2 < 2; ++h2) {
-            const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+        for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+            const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
             const bool on = s < L.g.V;
             C<double> acc[6], p[6];
             hop64_half<RECON, false>(L, L.x, s, hh, on, acc);
@@ -248,8 +257,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
         const SiteHalf pt{hh};
         const bool nz = a.lstate[2 * l] != 0;
         double v[1] = {0.0};
-        for (int h2 = 0; h2 < 2; ++h2) {
-            const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+        for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+            const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
             const bool on = s < L.g.V;
             C<double> acc[6], q[6], d[6];
             hop64_half<RECON, true>(L, L.t, s, hh, on && nz, acc);
@@ -279,8 +288,7 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
     });
     if (!grid_barrier(a)) return;
     // S4: rs = ps = r (inner precision) ; xs = 0
-    for_tiles(a, all, [&](const LatDesc &L, int, int, int s, bool valid) {
-        if (!valid) return;
+    for_tiles(a, all, [&](const LatDesc &L, int, int s) {
         C<double> d[12];
         SpinorIO<F64>::template load<false>(L.r, L.g.Vs, s, d);
         C<RS> w[12];
@@ -293,7 +301,7 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
         SpinorIO<SP>::store(L.rs, L.g.Vs, s, w);
         SpinorIO<SP>::store(L.ps, L.g.Vs, s, w);
         SpinorIO<F32>::store(L.xs, L.g.Vs, s, z);
-    });
+    }, none);
     if (!grid_barrier(a)) return;
 
     for (int it = 0; it < a.max_iter + 2; ++it) {
@@ -302,16 +310,15 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
         if (!any) break;
         if (threadIdx.x == 0 && blockIdx.x == 0) a.flags[2] = it + 1;
         // A: ts = D ps ; pAp = |ts|^2 ; alpha
-        for_tiles(a, active, [&](const LatDesc &L, int g, int l, int s, bool valid) {
-            double v[1] = {0.0};
-            if (valid) {
-                C<RS> acc[12], p[12];
-                hopping<SP, RIN, false, false>(L.g, L.ps, L.gs, L.gdirs, s, acc);
-                SpinorIO<SP>::template load<false>(L.ps, L.g.Vs, s, p);
-                xpay_site(p, acc, RS(L.kappa));
-                v[0] = norm2_of(p);
-                SpinorIO<SP>::store(L.ts, L.g.Vs, s, p);
-            }
+        double v[1] = {0.0};
+        for_tiles(a, active, [&](const LatDesc &L, int, int s) {
+            C<RS> acc[12], p[12];
+            hopping<SP, RIN, false, false>(L.g, L.ps, L.gs, L.gdirs, s, acc);
+            SpinorIO<SP>::template load<false>(L.ps, L.g.Vs, s, p);
+            xpay_site(p, acc, RS(L.kappa));
+            v[0] += norm2_of(p);
+            SpinorIO<SP>::store(L.ts, L.g.Vs, s, p);
+        }, [&](const LatDesc &L, int g, int l) {
             tile_reduce<1>(a, L, g, l, v, [&](int l2, const double *t) {
                 Scalars &c = a.sc[l2];
                 c.pAp = t[0];
@@ -319,30 +326,29 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
                 else if (!(t[0] > 0.0)) { c.status = WD_ERR_BREAKDOWN; c.active = 0; }
                 else c.alpha = c.rho / t[0];
             });
+            v[0] = 0.0;
         });
         if (!grid_barrier(a)) return;
         // B: q = D^dag ts ; rs -= alpha q ; xs += alpha ps ; rho' = |rs|^2 ; decide
-        for_tiles(a, active, [&](const LatDesc &L, int g, int l, int s, bool valid) {
-            double v[1] = {0.0};
-            if (valid) {
-                const RS alpha = RS(a.sc[l].alpha);
-                C<RS> acc[12], q[12], w[12];
-                hopping<SP, RIN, true, false>(L.g, L.ts, L.gs, L.gdirs, s, acc);
-                SpinorIO<SP>::template load<false>(L.ts, L.g.Vs, s, q);
-                xpay_site(q, acc, RS(L.kappa));
-                SpinorIO<SP>::template load<false>(L.rs, L.g.Vs, s, w);
+        for_tiles(a, active, [&](const LatDesc &L, int l, int s) {
+            const RS alpha = RS(a.sc[l].alpha);
+            C<RS> acc[12], q[12], w[12];
+            hopping<SP, RIN, true, false>(L.g, L.ts, L.gs, L.gdirs, s, acc);
+            SpinorIO<SP>::template load<false>(L.ts, L.g.Vs, s, q);
+            xpay_site(q, acc, RS(L.kappa));
+            SpinorIO<SP>::template load<false>(L.rs, L.g.Vs, s, w);
 #pragma unroll
-                for (int c = 0; c < 12; ++c) w[c] = C<RS>{w[c].re - alpha * q[c].re, w[c].im - alpha * q[c].im};
-                v[0] = norm2_of(w);
-                SpinorIO<SP>::store(L.rs, L.g.Vs, s, w);
-                SpinorIO<SP>::template load<false>(L.ps, L.g.Vs, s, q);
-                C<float> xs[12];
-                SpinorIO<F32>::template load<false>(L.xs, L.g.Vs, s, xs);
+            for (int c = 0; c < 12; ++c) w[c] = C<RS>{w[c].re - alpha * q[c].re, w[c].im - alpha * q[c].im};
+            v[0] += norm2_of(w);
+            SpinorIO<SP>::store(L.rs, L.g.Vs, s, w);
+            SpinorIO<SP>::template load<false>(L.ps, L.g.Vs, s, q);
+            C<float> xs[12];
+            SpinorIO<F32>::template load<false>(L.xs, L.g.Vs, s, xs);
 #pragma unroll
-                for (int c = 0; c < 12; ++c)
-                    xs[c] = C<float>{xs[c].re + float(alpha * q[c].re), xs[c].im + float(alpha * q[c].im)};
-                SpinorIO<F32>::store(L.xs, L.g.Vs, s, xs);
-            }
+            for (int c = 0; c < 12; ++c)
+                xs[c] = C<float>{xs[c].re + float(alpha * q[c].re), xs[c].im + float(alpha * q[c].im)};
+            SpinorIO<F32>::store(L.xs, L.g.Vs, s, xs);
+        }, [&](const LatDesc &L, int g, int l) {
             tile_reduce<1>(a, L, g, l, v, [&](int l2, const double *t) {
                 Scalars &c = a.sc[l2];
                 const double rn = t[0];
@@ -363,12 +369,12 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
                     if (c.pending && c.iter - c.pending_since >= kDeferIters) atomicExch(a.flags + 1, 1);
                 }
             });
+            v[0] = 0.0;
         });
         if (!grid_barrier(a)) return;
         if (*(volatile int *)(a.flags + 1)) {
             // C1: x += xs ; xs = 0  (FP64 solution accumulation)
-            for_tiles(a, updating, [&](const LatDesc &L, int, int, int s, bool valid) {
-                if (!valid) return;
+            for_tiles(a, updating, [&](const LatDesc &L, int, int s) {
                 C<double> x[12];
                 C<float> xs[12];
                 SpinorIO<F64>::template load<false>(L.x, L.g.Vs, s, x);
@@ -380,14 +386,14 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
                 }
                 SpinorIO<F64>::store(L.x, L.g.Vs, s, x);
                 SpinorIO<F32>::store(L.xs, L.g.Vs, s, xs);
-            });
+            }, none);
             if (!grid_barrier(a)) return;
             // C2: t = D x (FP64) ; |b - t|^2 (the final check's first norm, should x stay)
             for_tiles_half(a, updating, [&](const LatDesc &L, int g, int l, int sl, int hh) {
                 const SiteHalf pt{hh};
                 double v[1] = {0.0};
-                for (int h2 = 0; h2 < 2; ++h2) {
-                    const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+                for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+                    const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
                     const bool on = s < L.g.V;
                     C<double> acc[6], p[6], bb[6];
                     hop64_half<RECON, false>(L, L.x, s, hh, on, acc);
@@ -408,8 +414,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
             for_tiles_half(a, updating, [&](const LatDesc &L, int g, int l, int sl, int hh) {
                 const SiteHalf pt{hh};
                 double v[1] = {0.0};
-                for (int h2 = 0; h2 < 2; ++h2) {
-                    const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+                for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+                    const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
                     const bool on = s < L.g.V;
                     C<double> acc[6], q[6], d[6];
                     hop64_half<RECON, true>(L, L.t, s, hh, on, acc);
@@ -445,8 +451,7 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
             if (!grid_barrier(a)) return;
         }
         // D: rs = r (after a reliable update) ; ps = rs + beta ps
-        for_tiles(a, active, [&](const LatDesc &L, int, int l, int s, bool valid) {
-            if (!valid) return;
+        for_tiles(a, active, [&](const LatDesc &L, int l, int s) {
             const Scalars &c = a.sc[l];
             const RS beta = RS(c.beta);
             C<RS> w[12], p[12];
@@ -463,7 +468,7 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
 #pragma unroll
             for (int k = 0; k < 12; ++k) p[k] = C<RS>{w[k].re + beta * p[k].re, w[k].im + beta * p[k].im};
             SpinorIO<SP>::store(L.ps, L.g.Vs, s, p);
-        });
+        }, none);
         if (!grid_barrier(a)) return;
         // clear the pending flags (one block owns them), then a barrier before the next step
         if (blockIdx.x == 0) {
@@ -483,8 +488,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
     for_tiles_half(a, unchecked, [&](const LatDesc &L, int g, int l, int sl, int hh) {
         const SiteHalf pt{hh};
         double v[1] = {0.0};
-        for (int h2 = 0; h2 < 2; ++h2) {
-            const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+        for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+            const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
             const bool on = s < L.g.V;
             C<double> acc[6], p[6], bb[6];
             hop64_half<RECON, false>(L, L.x, s, hh, on, acc);
@@ -504,8 +509,8 @@ __global__ void __launch_bounds__(kTile, 5) k_batched_cg(BatchArgs a) {
     for_tiles_half(a, unchecked, [&](const LatDesc &L, int g, int l, int sl, int hh) {
         const SiteHalf pt{hh};
         double v[1] = {0.0};
-        for (int h2 = 0; h2 < 2; ++h2) {
-            const int s = (g - L.tile0) * kTile + h2 * kHalfTile + sl;
+        for (int h2 = 0; h2 < a.tile / kHalfTile; ++h2) {
+            const int s = (g - L.tile0) * a.tile + h2 * kHalfTile + sl;
             const bool on = s < L.g.V;
             C<double> acc[6], q[6], d[6];
             hop64_half<RECON, true>(L, L.t, s, hh, on, acc);
@@ -528,7 +533,7 @@ template <int SP, int RECON, int RIN>
 static cudaError_t build_batched(BatchArgs &a, cudaGraphExec_t *exec) {
     auto k = k_batched_cg<SP, RECON, RIN>;
     int per_sm = 0, dev = 0, sms = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kTile, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, 0);
     if (e != cudaSuccess) return e;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -537,7 +542,7 @@ static cudaError_t build_batched(BatchArgs &a, cudaGraphExec_t *exec) {
     if (grid < 1) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kTile);
+    cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = 0;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -582,6 +587,9 @@ extern "C" wd_status wd_cg_solve_batched(wd_ctx *const *ctxs, const double *kapp
     std::vector<LatDesc> lat(n);
     std::vector<int> tile_lat;
     int ntiles = 0;
+    long long sites = 0;
+    for (int i = 0; i < n; ++i) sites += ctxs[i] ? ctxs[i]->g.V : 0;
+    const int tile = tile_sites(sites);
     for (int i = 0; i < n; ++i) {
         wd_ctx *c = ctxs[i];
         if (!c || !b[i] || !x[i] || !std::isfinite(kappas[i]))
@@ -615,7 +623,7 @@ extern "C" wd_status wd_cg_solve_batched(wd_ctx *const *ctxs, const double *kapp
         if ((s = ws_get(c, "bt_xs", f32, &L.xs)) != WD_OK) return fail(c0, s, c->last_error);
         L.b = const_cast<void *>(b[i]);
         L.tile0 = ntiles;
-        L.ntiles = (c->g.V + kTile - 1) / kTile;
+        L.ntiles = (c->g.V + tile - 1) / tile;
         ntiles += L.ntiles;
         tile_lat.insert(tile_lat.end(), L.ntiles, i);
     }
@@ -655,6 +663,7 @@ extern "C" wd_status wd_cg_solve_batched(wd_ctx *const *ctxs, const double *kapp
     a.tpart = (double *)d_part;
     a.tile_lat = (const int *)d_tl;
     a.ntiles = ntiles;
+    a.tile = tile;
     a.nlat = n;
     a.max_iter = prm->max_iter;
     a.bar_count = (unsigned *)d_bar;
@@ -671,7 +680,7 @@ extern "C" wd_status wd_cg_solve_batched(wd_ctx *const *ctxs, const double *kapp
         return fail(c0, WD_ERR_ARG, "wd_cg_solve_batched: with compressed FP64 links the inner precision needs the "
                                     "same compression");
     char key[160];
-    snprintf(key, sizeof key, "batch|%d|%d,%d|%d|%d|%d|%d|%p|%p", (int)sp, r64, rin, n, ntiles, prm->max_iter,
+    snprintf(key, sizeof key, "batch|%d|%d,%d|%d|%d,%d|%d|%d|%p|%p", (int)sp, r64, rin, n, ntiles, tile, prm->max_iter,
              a.stall_test, d_part, d_lat);
     cudaGraphExec_t exec = (cudaGraphExec_t)graph_get(c0, key);
     if (!exec) {

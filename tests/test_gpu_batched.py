@@ -193,3 +193,31 @@ def test_batched_full_c5_workload(wd, rin):
         x_ref, _ = oracle.cgnr(U, b, kappas[i], dims, tol=1e-13)
         assert oracle.rel_err(lats[i].unpack(xs[i]), x_ref) < 1e-9, (i, dims)
     assert len({r["iters"] for r in res}) > 1
+
+
+def test_a_batch_large_enough_for_two_sites_per_thread(wd):
+    """From 4 x 256 x the resident blocks sites on a tile holds two sites per thread; volumes that
+    are no multiple of a tile, against the same lattices solved alone."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(3)
+    small = gen.haar_links((4, 4, 4, 4), seed=9)
+    shapes = [(16, 16, 16, 16)] * 12 + [(15, 13, 7, 5), (6, 5, 7, 9)]
+    lats, bs, xs = [], [], []
+    for dims in shapes:
+        V = int(np.prod(dims))
+        idx = torch.randint(256, (4, V), generator=g, device="cuda")
+        U = torch.from_numpy(small).cuda()
+        U = torch.stack([U[mu][idx[mu]] for mu in range(4)])
+        b = torch.complex(*[torch.randn(V, 4, 3, generator=g, device="cuda", dtype=torch.float64) for _ in range(2)])
+        lat = wd.Lattice(dims)
+        lat.set_gauge(U)
+        lats.append(lat)
+        bs.append(lat.pack(b))
+        xs.append(lat.new_field())
+    kappas = [0.11] * len(shapes)
+    res, st = wd.cg_batched(lats, kappas, bs, xs, tol=1e-10, inner=1)
+    assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
+    for i in (0, 11, 12, 13):
+        x1 = lats[i].new_field()
+        lats[i].cg(kappas[i], bs[i], x1, tol=1e-10, inner=1)
+        assert oracle.rel_err(lats[i].unpack(xs[i]), lats[i].unpack(x1)) < 1e-9
