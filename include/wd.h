@@ -122,8 +122,8 @@ wd_status wd_debug_word(wd_ctx *ctx, unsigned *word, int *is_debug);
 
 /* Store the links of one precision with another compression than wd_set_gauge's
  * (18, 12 or 8, with the recon = 8 condition above).  No counterpart in the paper: on
- * GB300 the FP64 operator is bound by the FP64 units, so compressed links only add
- * arithmetic there, while the FP32/FP16 operators are bound by memory and gain from
+ * GB300 the FP64 operator is bound by arithmetic, so compressed links only add to it
+ * there, while the FP32/FP16 operators are bound by memory and gain from
  * them; a mixed-precision solve can keep FP64 links whole (18) and compress the inner
  * precision's (12).  Applies until the next wd_set_gauge, which resets every precision
  * to its recon.  The solvers (wd_cg_solve* and wd_cg_solve_batched) accept any
@@ -406,8 +406,8 @@ wd_status wd_cg_solve_split(wd_ctx *const *ctxs, int n, double kappa, const void
 /* Measured FP64 arithmetic rate of the current device, in GFLOP/s (2 flop per fused
  * multiply-add): independent FP64 multiply-add chains on every SM, no memory traffic,
  * timed with CUDA events on a stream of its own (best of five launches after one
- * warm-up).  No counterpart in the paper: on GB300 the FP64 Dslash is bound by the
- * FP64 units, and this is the roof it is reported against.  Synchronises that stream;
+ * warm-up).  No counterpart in the paper: the rate of the FP64 pipe, beside which the
+ * FP64 Dslash, whose products run on other pipes, is reported.  Synchronises that stream;
  * changes no device setting.  Errors: WD_ERR_ARG (null), WD_ERR_CUDA. */
 wd_status wd_measure_fp64_rate(double *gflops);
 

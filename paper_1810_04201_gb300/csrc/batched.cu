@@ -11,7 +11,7 @@
 // lattice's scalar recursion, so every phase needs exactly one barrier.
 // Converged lattices drop out of the list; the kernel ends when none is left.
 // The FP64 phases (setup, reliable updates, final check) run two lanes per site
-// with paired hops, like the FP64 Dslash kernel; a zero start vector skips the
+// like the FP64 Dslash kernel; a zero start vector skips the
 // setup's D x0 and D^dag D x0; a reliable update that stops a lattice doubles as
 // its final check.
 //

@@ -1,6 +1,6 @@
-// FP64 arithmetic rate of the device: the roof of the FP64 Dslash on GPUs whose
-// FP64 units, not memory, bound that kernel (GB300 runs 2 FP64 FMAs per SM per
-// clock, so 1320 flop per 960 bytes needs far less than the HBM bandwidth).
+// FP64 arithmetic rate of the device.  GB300 runs 2 FP64 FMAs per SM per clock, so
+// 1320 flop per 960 bytes on the FP64 pipe would need far less than the HBM bandwidth;
+// the FP64 Dslash, whose products run on other pipes, is reported beside this rate.
 //
 // Every thread runs kChains independent multiply-add chains acc = acc * m + c,
 // so the FP64 pipe always has independent work; there are no memory accesses in
