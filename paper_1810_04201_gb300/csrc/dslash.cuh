@@ -1063,9 +1063,11 @@ __device__ __forceinline__ void store_part(const Pt &pt, void *base, int Vs, int
 // 10.3 -> 8.3 at 16^4 (four blocks: 64 registers, spills, 305 us; one: 215 registers, 235 us).
 // The FP64 hops wait on results of the integer and FP64 pipes and are held to 128 registers
 // (32^3 x 64: 811-850 us; 112 registers 841-848, 96 827-833 and slower on small lattices);
-// DF32 is arithmetic-bound and keeps the compiler's choice.
+// DF32 likewise: left alone, the solver epilogues take 134 (one block of 64 x 4 threads per SM,
+// 12 right-hand sides at 24^3 x 48 537 ms a solve against 408) and recon-12 more (24^3 x 48 431 /
+// 325 us, 16^3 x 32 87 / 74).
 template <int P, int RECON> constexpr int dslash_min_blocks() {
-    return P == F64 || (P == F32 && RECON == 18) ? 2 : P == F32 || P == F16 ? 3 : 0;
+    return P == F64 || P == DF32 || (P == F32 && RECON == 18) ? 2 : 3;
 }
 
 // Site tile (tile_x, in [0, gridDim.x)) and right-hand-side group (tile_y, in

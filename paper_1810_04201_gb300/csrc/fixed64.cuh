@@ -17,8 +17,8 @@
 // Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 811-850 us (128- and 64-thread blocks),
 // 16^4 107 -> 34.5 us; with recon-12 links 5066 -> 1083 us.  (Three integer products of 29-bit
 // limbs per real product, the first form: 882-888, 36.5 and 1400 us.)  What bounds it now is the
-// latency of its integer and FP64 results with 16 warps per SM: the integer and multiply-add pipes
-// are busy 41 and 37 % of the cycles, FP64 37 %, DRAM 20 %.
+// latency of its integer and FP64 results with 16 warps per SM: on 32^3 x 64 the integer, multiply-
+// add and FP64 pipes are busy 47, 39 and 38 % of the cycles, DRAM 32 %, issue slots 50 %.
 //
 // Bounds.  A spinor component is a sum of two doubles, each below (1 - 2^-21) units, so H fits 32
 // bits; |L| <= 2^31; links |H| <= 2^30 (1 + 2^-11) with rows and columns of norm at most
