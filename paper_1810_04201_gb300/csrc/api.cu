@@ -203,7 +203,8 @@ void graph_clear(wd_ctx *c) {
 // 130.8 with two per block; the plain operators differ, see tiles_for).  FP32 rows go in pairs on
 // one thread from 2^17 site-rows on with four rows (24^3 x 48: 41.3 -> 39.6 ms) and, even-odd, with
 // more (20^3 x 40, 12 rows 37.9 -> 36.3); two rows gain nothing (21.2 / 21.7 ms), and 12 rows on the
-// whole lattice lose (126 / 134 ms).
+// whole lattice lose (126 / 134 ms).  With recon-12 links the pairs still gain (four rows at
+// 16^3 x 32 even-odd 6.13 -> 5.65 ms, at 24^4 19.6 -> 19.1), with recon-8 they lose (24^3 x 48 37.5 / 40.0).
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
     if (it != c->cg_tiles.end()) return it->second;
@@ -217,7 +218,8 @@ DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     t.site_tile = 64;
     t.rhs_tile = nrhs < 4 ? nrhs : 4;
     const long long work = (long long)c->g.V * nrhs / (eo ? 2 : 1);
-    if (p == F32 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) && work >= (1 << 17)) t.rhs_per_thread = 2;
+    if (p == F32 && link_recon(c, p) != 8 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) && work >= (1 << 17))
+        t.rhs_per_thread = 2;
     return t;
 }
 
@@ -234,8 +236,11 @@ void ws_release(wd_ctx *c, const std::string &name) {
 // per block: the blocks of a site tile's right-hand sides start together and share its links
 // through L2, and a block's rows leave no idle threads when nrhs is odd (24^3 x 48, 64 x 1
 // against 64 x 4, us: FP32 12 rows 586 / 618, 7 rows 339 / 388; FP16 408 / 438, 241 / 277).
-// FP32 rows in pairs on one thread from 2^17 site-rows on (12 rows 562, 4 rows 186 / 200; at
-// 8^3 x 16 with two rows 8.5 / 6.7).  Larger blocks for FP64 from 2^18 site-rows on (256 / 64
+// FP32 rows with whole links go in pairs on one thread, each link loaded once for both, from 2^17
+// site-rows on, two rows from 2^20 on (pairs / 64 x 1, us: 12 rows 569 / 608, 4 rows 190 / 206,
+// 4 rows at 16^4 24.1 / 25.0; two rows 106 / 110, at 28^4 99 / 105, at 24^4 59.4 / 58.9, at 20^4
+// 35.2 / 33.2).  Compressed links are few enough that the pairs' lower occupancy costs more
+// (recon-12: 12 rows 571 / 539, two rows at 20^4 33.1 / 29.0).  Larger blocks for FP64 from 2^18 site-rows on (256 / 64
 // threads: 12 rows 3144 / 3289, one row at 32^3 x 64 838 / 876, at 16^4 38.6 / 36.4) and DF32
 // (128 / 64: 2810 / 2861).
 DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs) {
@@ -245,7 +250,8 @@ DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs) {
     DslashTiles t;
     t.site_tile = p == DF32 ? 128 : p == F64 && work >= (1 << 18) ? 256 : 64;
     t.rhs_tile = 1;
-    if (p == F32 && nrhs % 2 == 0 && work >= (1 << 17) && !c->split) t.rhs_tile = t.rhs_per_thread = 2;
+    if (p == F32 && link_recon(c, p) == 18 && nrhs % 2 == 0 && work >= (nrhs == 2 ? 1 << 20 : 1 << 17) && !c->split)
+        t.rhs_tile = t.rhs_per_thread = 2;
     return t;
 }
 
