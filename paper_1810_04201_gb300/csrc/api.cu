@@ -205,6 +205,11 @@ void graph_clear(wd_ctx *c) {
 // more (20^3 x 40, 12 rows 37.9 -> 36.3); two rows gain nothing (21.2 / 21.7 ms), and 12 rows on the
 // whole lattice lose (126 / 134 ms).  With recon-12 links the pairs still gain (four rows at
 // 16^3 x 32 even-odd 6.13 -> 5.65 ms, at 24^4 19.6 -> 19.1), with recon-8 they lose (24^3 x 48 37.5 / 40.0).
+// FP64 takes one row per block, which shares links through L2 as well and wastes no lanes: blocks of
+// 256 threads from 2^17 sites on (64 / 256, ms a solve: 16^3 x 32 24.8 / 23.0, 24^3 x 48 113.9 / 105.1,
+// even-odd 39.5 / 38.3, 12 rows 1255 (64 x 4) / 1237), 128 below with several rows (64 x 4 / 128 x 1,
+// four rows: 8^3 x 16 9.15 / 8.33, 16^3 x 32 even-odd 30.6 / 29.0; 256 x 1 at 12^3 x 24 30.9 against
+// 29.0); single rows below keep 64 (128: -7 to +3 %, by how the last wave fills).
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
     if (it != c->cg_tiles.end()) return it->second;
@@ -217,7 +222,11 @@ DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     }
     t.site_tile = 64;
     t.rhs_tile = nrhs < 4 ? nrhs : 4;
-    const long long work = (long long)c->g.V * nrhs / (eo ? 2 : 1);
+    const long long sites = c->g.V / (eo ? 2 : 1), work = sites * nrhs;
+    if (p == F64 && (nrhs > 1 || sites >= (1 << 17))) {
+        t.site_tile = sites >= (1 << 17) ? 256 : 128;
+        t.rhs_tile = 1;
+    }
     if (p == F32 && link_recon(c, p) != 8 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) && work >= (1 << 17))
         t.rhs_per_thread = 2;
     return t;
