@@ -808,6 +808,9 @@ __device__ __forceinline__ void fx_raise(FxAcc &acc, int e) {
 template <int RECON, bool DAG, int MU, bool ADJ, bool NC>
 __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs, int n, int sl, int hh, bool flip,
                                        bool zero, FxAcc &acc) {
+    // a hop that leaves a sub-lattice: n is the other end of the block and no neighbour, and must not
+    // set the unit either
+    if (MU == 3 && zero) return;
     constexpr bool IM = MU == 0 || MU == 2;         // f = +-i: the parts of psi_ps swap
     constexpr int SM = DAG != ADJ ? 0 : -1;         // sign masks: of S,
     constexpr int LO = 6;
@@ -851,13 +854,6 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
         } else {
             fx_sum(ph[c].re, fl, ar, mr ^ fl, cc, H[2 * c], L[2 * c]);
             fx_sum(ph[c].im, fl, ai, mi ^ fl, cc, H[2 * c + 1], L[2 * c + 1]);
-        }
-    }
-    if (MU == 3 && zero) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            H[k] = 0;
-            L[k] = 0.f;
         }
     }
     int4 u[9];

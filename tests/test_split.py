@@ -251,6 +251,32 @@ def test_split_cg_matches_oracle_solution(wd, dims, nranks):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dims,nranks,decades", [((4, 4, 4, 8), 2, 7), ((4, 2, 6, 6), 3, 20), ((5, 3, 4, 8), 8, 15)])
+@pytest.mark.parametrize("recon", [18, 12])
+def test_split_field_that_decays_along_t(wd, dims, nranks, decades, recon):
+    """The site across a cut in the rank's own block is no neighbour: a field that falls by
+    10^-decades from slice to slice, so that the two ends of a block differ by up to 1e-21 and more,
+    site by site against the unsplit oracle, within 2e-15 of the largest component that the site
+    and its true neighbours hold (the bound of the limb arithmetic, see test_gpu_fixed64.py)."""
+    kappa = 0.12
+    U = gen.haar_links(dims, seed=91)
+    vf = dims[0] * dims[1] * dims[2]
+    scale = np.repeat(10.0 ** (-decades * np.arange(dims[3], dtype=float)), vf)
+    psi = gen.gaussian_source(dims, seed=92) * scale[:, None, None]
+    big = np.abs(psi.view(np.float64)).reshape(*dims[::-1], -1).max(-1)
+    near = big.copy()
+    for ax in range(4):
+        near = np.maximum(near, np.maximum(np.roll(big, 1, ax), np.roll(big, -1, ax)))
+    blocks = split_blocks(wd, dims, nranks, U, recon=recon)
+    fields = [b.pack(b.split.local_field(psi, r)) for r, b in enumerate(blocks)]
+    for dagger in (False, True):
+        outs = split_apply(blocks, kappa, fields, 0, dagger)
+        got = np.concatenate([b.unpack(o) for b, o in zip(blocks, outs)])
+        want = oracle.apply_D(U, psi, kappa, dims, dagger=dagger)
+        assert np.all(np.abs(got - want).reshape(len(psi), -1).max(1) <= 2e-15 * near.reshape(-1))
+
+
+@pytest.mark.gpu
 def test_split_refusals(wd):
     dims = (4, 4, 4, 8)
     U = gen.haar_links(dims, seed=77)
