@@ -39,9 +39,10 @@
  * Ownership and streams.  The caller owns every field and canonical buffer; the
  * context owns its gauge copies, its workspace and its CUDA graphs, and frees
  * them in wd_destroy.  Every call is asynchronous on the context's stream, except
- * the solvers, which wait for the result to fill wd_cg_result, and the calls
+ * the solvers, which wait for the result to fill wd_cg_result, the calls
  * whose on_device flag is 0 (host buffers), which return once the host buffer
- * may be reused.
+ * may be reused, and wd_set_gauge, which waits for earlier work and for its check
+ * of the links (the FP64 copy alone is still being written when it returns).
  *
  * Errors.  Every call returns a status and never aborts or throws.  Argument
  * checks (null pointers, dimensions < 2, nrhs outside 1..WD_MAX_RHS, unknown
@@ -92,7 +93,12 @@ typedef struct wd_ctx wd_ctx;
 /* Create a context for an Lx x Ly x Lz x Lt lattice (dims[0..3], each >= 2) on the
  * current CUDA device.  stream is a cudaStream_t (NULL = the legacy default stream);
  * all work of this context is queued on it.  antiperiodic_t selects the antiperiodic
- * time boundary (section 2.3). */
+ * time boundary (section 2.3).
+ *
+ * wd_set_stream moves the context to another stream.  Work queued on the earlier one is not
+ * ordered before what follows on the new one (the caller orders them, e.g. by an event);
+ * only the calls that replace links, wd_set_gauge on a context that holds some and
+ * wd_set_link_compression, wait for all work on the device first. */
 wd_status wd_create(wd_ctx **ctx, const int dims[4], int antiperiodic_t, void *stream);
 wd_status wd_destroy(wd_ctx *ctx);
 wd_status wd_set_stream(wd_ctx *ctx, void *stream);

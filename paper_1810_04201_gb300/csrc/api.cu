@@ -359,7 +359,9 @@ wd_status wd_set_gauge(wd_ctx *c, const double *U, int on_device, int recon) {
     if (!U) return fail(c, WD_ERR_ARG, "wd_set_gauge: null gauge pointer");
     if (recon != 18 && recon != 12 && recon != 8) return fail(c, WD_ERR_ARG, "wd_set_gauge: recon must be 18, 12 or 8");
     const size_t bytes = (size_t)4 * c->g.V * 9 * 16;
-    WD_CUDA(c, cudaStreamSynchronize(c->stream));
+    // The links are replaced in place, and operators or solves that read them may be under way on a
+    // stream that this context (or a batch it took part in, or a captured graph) used before.
+    WD_CUDA(c, c->gauge_canon ? cudaDeviceSynchronize() : cudaStreamSynchronize(c->stream));
     // the copies are written again when next needed, in place (16^3 x 32, new links and an FP32
     // solve from host buffers: 4.97 ms with them freed, allocated and the solver's graph rebuilt
     // each time, 4.57 ms without)
@@ -409,7 +411,7 @@ wd_status wd_set_link_compression(wd_ctx *c, wd_prec prec, int recon) {
         wd_status s = check_recon8(c, "wd_set_link_compression");
         if (s != WD_OK) return s;
     }
-    WD_CUDA(c, cudaStreamSynchronize(c->stream));
+    WD_CUDA(c, cudaDeviceSynchronize());  // as in wd_set_gauge: the copies are refilled in place
     c->gauge_ok[prec] = c->gauge_eo_ok[prec] = false;
     c->recon_p[prec] = recon;
     return WD_OK;

@@ -53,3 +53,31 @@ def test_a_stale_copy_is_refused_where_a_missing_one_is():
         assert e.value.status == 8
         lat.apply(KAPPA, f, o, 1)
         lat.normal_apply_noalloc(KAPPA, f, o, 1)
+
+
+@pytest.mark.parametrize("on_device", [False, True])
+def test_new_links_wait_for_operators_on_an_earlier_stream(on_device):
+    """Operators queued on the stream that a context used before must still see the old links."""
+    import torch
+    from paper_1810_04201_gb300 import wd
+    dims = (8, 8, 8, 12)
+    U1, U2 = gen.haar_links(dims, seed=1), gen.haar_links(dims, seed=2)
+    if on_device:
+        U2 = torch.from_numpy(U2).cuda()
+    src = gen.gaussian_source(dims, seed=3)
+    one, two = torch.cuda.Stream(), torch.cuda.Stream()
+    for prec in (0, 1):
+        with torch.cuda.stream(one):
+            lat = wd.Lattice(dims)
+            lat.set_gauge(U1)
+            f, want, got = lat.pack(src, prec), lat.new_field(prec), lat.new_field(prec)
+            lat.apply(KAPPA, f, want, prec)
+            one.synchronize()
+            torch.cuda._sleep(200_000_000)  # about a tenth of a second before the operator starts
+            lat.apply(KAPPA, f, got, prec)
+        with torch.cuda.stream(two):
+            lat.set_stream()
+            lat.set_gauge(U2)
+            lat.apply(KAPPA, f, lat.new_field(prec), prec)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
