@@ -808,9 +808,6 @@ __device__ __forceinline__ void fx_raise(FxAcc &acc, int e) {
 template <int RECON, bool DAG, int MU, bool ADJ, bool NC>
 __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs, int n, int sl, int hh, bool flip,
                                        bool zero, FxAcc &acc) {
-    // a hop that leaves a sub-lattice: n is the other end of the block and no neighbour, and must not
-    // set the unit either
-    if (MU == 3 && zero) return;
     constexpr bool IM = MU == 0 || MU == 2;         // f = +-i: the parts of psi_ps swap
     constexpr int SM = DAG != ADJ ? 0 : -1;         // sign masks: of S,
     constexpr int LO = 6;
@@ -826,6 +823,10 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
         mx = fx_max(mx, ph[c].re, ph[c].im);
         mx = fx_max(mx, pd[c].re, pd[c].im);
     }
+    // a hop that leaves a sub-lattice: n is the other end of the block and no neighbour, and must not
+    // set the unit (its limbs, whatever they are then, are zeroed below)
+    const bool out = MU == 3 && zero;
+    if (out) mx = 0.f;
     // + 1: components stay below (1 - 2^-21) units, so that rounded limbs cannot overflow
     const int e = (int)((__float_as_uint(mx) + 1u) >> 20);
     if (e > acc.E) {
@@ -838,7 +839,7 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
         for (int c = 0; c < 3; ++c)
             any |= __double_as_longlong(ph[c].re) | __double_as_longlong(ph[c].im) | __double_as_longlong(pd[c].re) |
                    __double_as_longlong(pd[c].im);
-        if (any << 1) acc.bad = 1;
+        if (any << 1 && !out) acc.bad = 1;
     }
     const unsigned cc = ((unsigned)(acc.E + 2) << 21) | 0x1fffffu;
     int H[6];
@@ -854,6 +855,13 @@ __device__ __forceinline__ void fx_hop(const void *in, const char *gdir, int Vs,
         } else {
             fx_sum(ph[c].re, fl, ar, mr ^ fl, cc, H[2 * c], L[2 * c]);
             fx_sum(ph[c].im, fl, ai, mi ^ fl, cc, H[2 * c + 1], L[2 * c + 1]);
+        }
+    }
+    if (out) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            H[k] = 0;
+            L[k] = 0.f;
         }
     }
     int4 u[9];
