@@ -131,6 +131,9 @@ static wd_status check_unitary(wd_ctx *c) {
     return WD_OK;
 }
 
+// whether the FP64 kernels multiply limbs (dslash_kernel's FX form)
+static bool fx_links(const wd_ctx *c) { return c->g.links_fx && link_recon(c, F64) != 8; }
+
 Geom eo_geom(const wd_ctx *c, int parity) {
     Geom g = c->g;
     g.V = c->g.V / 2;
@@ -210,6 +213,8 @@ void graph_clear(wd_ctx *c) {
 // even-odd 39.5 / 38.3, 12 rows 1255 (64 x 4) / 1237), 128 below with several rows (64 x 4 / 128 x 1,
 // four rows: 8^3 x 16 9.15 / 8.33, 16^3 x 32 even-odd 30.6 / 29.0; 256 x 1 at 12^3 x 24 30.9 against
 // 29.0); single rows below keep 64 (128: -7 to +3 %, by how the last wave fills).
+// With FP64 arithmetic (fx_links) 64 x 1 everywhere (64 x 1 / 64 x 4 / 256 x 1, four rows: 8^3 x 12 5.77 /
+// 7.39 / 7.28, 16^3 x 32 82.1 / 84.3 / 81.5, even-odd 43.3 / 44.5 / 44.4).
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
     if (it != c->cg_tiles.end()) return it->second;
@@ -223,7 +228,9 @@ DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     t.site_tile = 64;
     t.rhs_tile = nrhs < 4 ? nrhs : 4;
     const long long sites = c->g.V / (eo ? 2 : 1), work = sites * nrhs;
-    if (p == F64 && (nrhs > 1 || sites >= (1 << 17))) {
+    if (p == F64 && !fx_links(c)) {
+        t.rhs_tile = 1;
+    } else if (p == F64 && (nrhs > 1 || sites >= (1 << 17))) {
         t.site_tile = sites >= (1 << 17) ? 256 : 128;
         t.rhs_tile = 1;
     }
@@ -251,13 +258,15 @@ void ws_release(wd_ctx *c, const std::string &name) {
 // 35.2 / 33.2).  Compressed links are few enough that the pairs' lower occupancy costs more
 // (recon-12: 12 rows 571 / 539, two rows at 20^4 33.1 / 29.0).  Larger blocks for FP64 from 2^18 site-rows on (256 / 64
 // threads: 12 rows 3144 / 3289, one row at 32^3 x 64 838 / 876, at 16^4 38.6 / 36.4) and DF32
-// (128 / 64: 2810 / 2861).
+// (128 / 64: 2810 / 2861).  With FP64 arithmetic (fx_links) 64 threads: more of them leave the FP64
+// units of an SM's schedulers unevenly loaded (64 / 256 threads: 24^4 510 / 522, recon-12 797 / 839,
+// recon-8 1886 / 1951).
 DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs) {
     auto it = c->tiles.find(p * 64 + nrhs);
     if (it != c->tiles.end()) return it->second;
     const long long work = (long long)c->g.V * nrhs;
     DslashTiles t;
-    t.site_tile = p == DF32 ? 128 : p == F64 && work >= (1 << 18) ? 256 : 64;
+    t.site_tile = p == DF32 ? 128 : p == F64 && fx_links(c) && work >= (1 << 18) ? 256 : 64;
     t.rhs_tile = 1;
     if (p == F32 && link_recon(c, p) == 18 && nrhs % 2 == 0 && work >= (nrhs == 2 ? 1 << 20 : 1 << 17) && !c->split)
         t.rhs_tile = t.rhs_per_thread = 2;

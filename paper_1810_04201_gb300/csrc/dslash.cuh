@@ -128,7 +128,7 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const void *in, const cha
         C<R> p[12], h[6], w[6], u[9];
         SpinorIO<P>::template load<NC>(in, g.Vs, sf, p);
         project<MU, SF>(p, h);
-        load_link<P, RECON>(g, gdir, g.Vs, s, u);
+        load_link<P, RECON>(gdir, g.Vs, s, u);
         su3_mult<false>(u, h, w, MU == 3 && g.antiperiodic && c == L - 1);
         if (MU == 3 && g.split_t && c == L - 1) zero6(w);  // the neighbour lives on the next sub-lattice
         accumulate<MU, SF>(acc, w);
@@ -138,7 +138,7 @@ __device__ __forceinline__ void hop_dir(const Geom &g, const void *in, const cha
         C<R> p[12], h[6], w[6], u[9];
         SpinorIO<P>::template load<NC>(in, g.Vs, sb, p);
         project<MU, -SF>(p, h);
-        load_link<P, RECON>(g, gdir, g.Vs, sb, u);
+        load_link<P, RECON>(gdir, g.Vs, sb, u);
         su3_mult<true>(u, h, w, MU == 3 && g.antiperiodic && c == 0);
         if (MU == 3 && g.split_t && c == 0) zero6(w);  // the neighbour lives on the previous sub-lattice
         accumulate<MU, -SF>(acc, w);
@@ -373,7 +373,7 @@ __device__ __forceinline__ void hop_dir_eo(const Geom &g, const void *in, const 
             C<R> p[12], h[6], w[6], u[9];
             SpinorIO<P>::template load<NC>(in, g.Vs, nf >> 1, p);
             project<MU, SF>(p, h);
-            load_link<P, RECON>(g, gp, g.Vs, k, u);
+            load_link<P, RECON>(gp, g.Vs, k, u);
             su3_mult<false>(u, h, w, MU == 3 && g.antiperiodic && c == L - 1);
             accumulate<MU, SF>(acc, w);
         }
@@ -382,7 +382,7 @@ __device__ __forceinline__ void hop_dir_eo(const Geom &g, const void *in, const 
             C<R> p[12], h[6], w[6], u[9];
             SpinorIO<P>::template load<NC>(in, g.Vs, nb >> 1, p);
             project<MU, -SF>(p, h);
-            load_link<P, RECON>(g, gq, g.Vs, nb >> 1, u);
+            load_link<P, RECON>(gq, g.Vs, nb >> 1, u);
             su3_mult<true>(u, h, w, MU == 3 && g.antiperiodic && c == 0);
             accumulate<MU, -SF>(acc, w);
         }
@@ -487,7 +487,7 @@ __device__ __forceinline__ void su3_mult1(const C<R> (&u)[9], const C<R> (&h)[3]
 // mu is a run-time value (constant-folded where the caller unrolls the directions);
 // LO = 3 for mu = 0, 1 and 6 for mu = 2, 3 selects the accumulator block of spin ps.
 
-template <int P, int RECON, bool DAG, int LO, bool NC, class R>
+template <int P, int RECON, bool DAG, int LO, bool NC, bool FX, class R>
 __device__ __forceinline__ void half_pair(const Geom &g, int mu, const void *in, int nf, const char *gf, int kf, bool flip_f,
                                           int nb, const char *gb, int kb, bool flip_b, int hh, C<R> (&acc)[9],
                                           bool zero_f = false, bool zero_b = false) {
@@ -507,7 +507,7 @@ __device__ __forceinline__ void half_pair(const Geom &g, int mu, const void *in,
             h[c] = cxsign(SF > 0 ? cadd(ph[c], fd) : csub(ph[c], fd), flip_f);
             if (zero_f) h[c] = C<R>{R(0), R(0)};
         }
-        load_link<P, RECON>(g, gf, Vs, kf, u);
+        load_link<P, RECON, FX>(gf, Vs, kf, u);
         su3_mult1<false>(u, h, wf);
     }
     {
@@ -520,7 +520,7 @@ __device__ __forceinline__ void half_pair(const Geom &g, int mu, const void *in,
             h[c] = cxsign(SF > 0 ? csub(ph[c], fd) : cadd(ph[c], fd), flip_b);
             if (zero_b) h[c] = C<R>{R(0), R(0)};
         }
-        load_link<P, RECON>(g, gb, Vs, kb, u);
+        load_link<P, RECON, FX>(gb, Vs, kb, u);
         // sum = w_f + U^dag h
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -538,24 +538,24 @@ __device__ __forceinline__ void half_pair(const Geom &g, int mu, const void *in,
     }
 }
 
-template <int P, int RECON, bool DAG, int MU, bool NC, class R>
+template <int P, int RECON, bool DAG, int MU, bool NC, bool FX, class R>
 __device__ __forceinline__ void half_dir(const Geom &g, const void *in, const char *gdir, int s, int c, int hh,
                                          C<R> (&acc)[9]) {
     const int L = g.L[MU], st = g.stride[MU];
     const int sf = WD_IDX(g, (c == L - 1) ? s - (L - 1) * st : s + st, g.V, 1);
     const int sb = WD_IDX(g, (c == 0) ? s + (L - 1) * st : s - st, g.V, 2);
-    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(g, MU, in, sf, gdir, s, MU == 3 && g.antiperiodic && c == L - 1,
+    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC, FX>(g, MU, in, sf, gdir, s, MU == 3 && g.antiperiodic && c == L - 1,
                                                 sb, gdir, sb, MU == 3 && g.antiperiodic && c == 0, hh, acc,
                                                 MU == 3 && g.split_t && c == L - 1, MU == 3 && g.split_t && c == 0);
 }
 
-template <int P, int RECON, bool DAG, int MU, bool NC, class R>
+template <int P, int RECON, bool DAG, int MU, bool NC, bool FX, class R>
 __device__ __forceinline__ void half_dir_eo(const Geom &g, const void *in, const char *gp, const char *gq, int k,
                                             int n, int c, int hh, C<R> (&acc)[9]) {
     const int L = g.L[MU], st = g.stride[MU];
     const int nf = WD_IDX(g, (c == L - 1) ? n - (L - 1) * st : n + st, 2 * g.V, 3);
     const int nb = WD_IDX(g, (c == 0) ? n + (L - 1) * st : n - st, 2 * g.V, 4);
-    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC>(g, MU, in, nf >> 1, gp, k, MU == 3 && g.antiperiodic && c == L - 1,
+    half_pair<P, RECON, DAG, MU < 2 ? 3 : 6, NC, FX>(g, MU, in, nf >> 1, gp, k, MU == 3 && g.antiperiodic && c == L - 1,
                                                 nb >> 1, gq, nb >> 1, MU == 3 && g.antiperiodic && c == 0, hh, acc);
 }
 
@@ -686,8 +686,9 @@ __device__ __forceinline__ void half_rolled(const Geom &g, const void *in, const
     }
 }
 
-// the hopping sum of lane half hh at site s (full lattice) or checkerboard index s (EO)
-template <int P, int RECON, bool DAG, bool EO, bool NC = true>
+// the hopping sum of lane half hh at site s (full lattice) or checkerboard index s (EO); FX: the
+// FP64 links are limbs
+template <int P, int RECON, bool DAG, bool EO, bool NC, bool FX>
 __device__ __forceinline__ void hopping_half(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                              int hh, C<typename Real<P>::T> (&acc)[9]) {
     using R = typename Real<P>::T;
@@ -720,18 +721,18 @@ __device__ __forceinline__ void hopping_half(const Geom &g, const void *in, cons
         const int n = eo_full_index(g, s, x, y, z, t);
         const char *gp = reinterpret_cast<const char *>(gauge) + (size_t)(4 * g.eo_parity) * gdir_bytes;
         const char *gq = reinterpret_cast<const char *>(gauge) + (size_t)(4 * (1 - g.eo_parity)) * gdir_bytes;
-        half_dir_eo<P, RECON, DAG, 0, NC>(g, in, gp, gq, s, n, x, hh, acc);
-        half_dir_eo<P, RECON, DAG, 1, NC>(g, in, gp + gdir_bytes, gq + gdir_bytes, s, n, y, hh, acc);
-        half_dir_eo<P, RECON, DAG, 2, NC>(g, in, gp + 2 * gdir_bytes, gq + 2 * gdir_bytes, s, n, z, hh, acc);
-        half_dir_eo<P, RECON, DAG, 3, NC>(g, in, gp + 3 * gdir_bytes, gq + 3 * gdir_bytes, s, n, t, hh, acc);
+        half_dir_eo<P, RECON, DAG, 0, NC, FX>(g, in, gp, gq, s, n, x, hh, acc);
+        half_dir_eo<P, RECON, DAG, 1, NC, FX>(g, in, gp + gdir_bytes, gq + gdir_bytes, s, n, y, hh, acc);
+        half_dir_eo<P, RECON, DAG, 2, NC, FX>(g, in, gp + 2 * gdir_bytes, gq + 2 * gdir_bytes, s, n, z, hh, acc);
+        half_dir_eo<P, RECON, DAG, 3, NC, FX>(g, in, gp + 3 * gdir_bytes, gq + 3 * gdir_bytes, s, n, t, hh, acc);
     } else {
         int x, y, z, t;
         site_xyzt(g, s, x, y, z, t);
         const char *gb = reinterpret_cast<const char *>(gauge);
-        half_dir<P, RECON, DAG, 0, NC>(g, in, gb, s, x, hh, acc);
-        half_dir<P, RECON, DAG, 1, NC>(g, in, gb + gdir_bytes, s, y, hh, acc);
-        half_dir<P, RECON, DAG, 2, NC>(g, in, gb + 2 * gdir_bytes, s, z, hh, acc);
-        half_dir<P, RECON, DAG, 3, NC>(g, in, gb + 3 * gdir_bytes, s, t, hh, acc);
+        half_dir<P, RECON, DAG, 0, NC, FX>(g, in, gb, s, x, hh, acc);
+        half_dir<P, RECON, DAG, 1, NC, FX>(g, in, gb + gdir_bytes, s, y, hh, acc);
+        half_dir<P, RECON, DAG, 2, NC, FX>(g, in, gb + 2 * gdir_bytes, s, z, hh, acc);
+        half_dir<P, RECON, DAG, 3, NC, FX>(g, in, gb + 3 * gdir_bytes, s, t, hh, acc);
     }
 }
 
@@ -755,8 +756,9 @@ template <class R> __device__ __forceinline__ void exchange_halves(C<R> (&acc)[9
 // power-of-two unit 2^(E - 1022): a hop whose spinors are larger than the unit raises it and
 // shifts the sums down.  The directions of a lower spin that goes to the partner lane come
 // first, so that a lane holds two spins of sums and not three.  FP64 arithmetic remains for half
-// of the projections, the final sums as doubles and for what this cannot take (recon-8 links,
-// links that are not unitary, non-finite, huge or tiny spinors), which goes through half_native.
+// of the projections, the final sums as doubles and for spinors that this cannot take (non-finite,
+// huge or tiny), whose sites go through half_native.  Recon-8 links and links that are not unitary
+// have kernels in FP64 arithmetic (dslash_kernel with FX = false).
 struct FxAcc {
     long long v[12];  // upper spin hh, then the lower spin under way: 3 x (re, im) each
     int E;            // the unit: 2^(E - 1022 - kFxAccBits)
@@ -941,38 +943,36 @@ __device__ __forceinline__ void fx_hopping(const Geom &g, const void *in, const 
 template <int RECON, bool DAG, bool EO, bool NC>
 __device__ __noinline__ void half_native(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                          int hh, C<double> (&acc)[9]) {
-    hopping_half<F64, RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+    hopping_half<F64, RECON, DAG, EO, NC, true>(g, in, gauge, gdir_bytes, s, hh, acc);
 }
 
 // The hopping sum of site s for the spins this lane owns (hh and 3 - hh), zero where `on` is
 // false.  Every lane of the warp calls it (on is the same for both lanes of a site).
-template <int P, int RECON, bool DAG, bool EO, bool NC = true>
+// FX: links as limbs (Geom::links_fx), with lanes that the limbs cannot take redone in FP64.
+template <int P, int RECON, bool DAG, bool EO, bool NC, bool FX>
 __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                             int hh, bool on, C<typename Real<P>::T> (&own)[6]) {
     using R = typename Real<P>::T;
-    if constexpr (P == F64 && RECON != 8) {
-        bool native = !g.links_fx;
-        if (!native) {
-            FxAcc acc;
+    if constexpr (FX) {
+        FxAcc acc;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) acc.v[k] = 0;
-            acc.E = kFxMinExp;
-            acc.bad = 0;
-            if (on) fx_hopping<RECON, DAG, EO, NC, 1>(g, in, gauge, gdir_bytes, s, hh, acc);
-            // both lanes in one unit; the partner's spin 2 + hh' is this lane's 3 - hh
-            const int Ep = __shfl_xor_sync(0xffffffffu, acc.E, 16);
-            if (Ep > acc.E) fx_raise(acc, Ep);
+        for (int k = 0; k < 12; ++k) acc.v[k] = 0;
+        acc.E = kFxMinExp;
+        acc.bad = 0;
+        if (on) fx_hopping<RECON, DAG, EO, NC, 1>(g, in, gauge, gdir_bytes, s, hh, acc);
+        // both lanes in one unit; the partner's spin 2 + hh' is this lane's 3 - hh
+        const int Ep = __shfl_xor_sync(0xffffffffu, acc.E, 16);
+        if (Ep > acc.E) fx_raise(acc, Ep);
 #pragma unroll
-            for (int k = 6; k < 12; ++k) acc.v[k] = __shfl_xor_sync(0xffffffffu, acc.v[k], 16);
-            if (on) fx_hopping<RECON, DAG, EO, NC, 0>(g, in, gauge, gdir_bytes, s, hh, acc);
-            const int e = acc.E - 1022 - kFxAccBits;
+        for (int k = 6; k < 12; ++k) acc.v[k] = __shfl_xor_sync(0xffffffffu, acc.v[k], 16);
+        if (on) fx_hopping<RECON, DAG, EO, NC, 0>(g, in, gauge, gdir_bytes, s, hh, acc);
+        const int e = acc.E - 1022 - kFxAccBits;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                own[k] = C<R>{fx_value(acc.v[2 * k], e), fx_value(acc.v[2 * k + 1], e)};
-                own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
-            }
-            native = acc.bad;
+        for (int k = 0; k < 3; ++k) {
+            own[k] = C<R>{fx_value(acc.v[2 * k], e), fx_value(acc.v[2 * k + 1], e)};
+            own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
         }
+        bool native = acc.bad;
         if (__any_sync(0xffffffffu, native)) {
             native |= __shfl_xor_sync(0xffffffffu, native, 16) != 0;
             C<double> acc[9];
@@ -986,7 +986,7 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
         }
     } else {
         C<R> acc[9];
-        if (on) hopping_half<P, RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
+        if (on) hopping_half<P, RECON, DAG, EO, NC, false>(g, in, gauge, gdir_bytes, s, hh, acc);
         else
 #pragma unroll
             for (int k = 0; k < 9; ++k) acc[k] = C<R>{R(0), R(0)};
@@ -1070,9 +1070,17 @@ __device__ __forceinline__ void store_part(const Pt &pt, void *base, int Vs, int
 // DF32 likewise: left alone, the solver epilogues take 134 (one block of 64 x 4 threads per SM,
 // 12 right-hand sides at 24^3 x 48 537 ms a solve against 408) and recon-12 more (24^3 x 48 431 /
 // 325 us, 16^3 x 32 87 / 74).
-template <int P, int RECON> constexpr int dslash_min_blocks() {
+template <int P, int RECON, bool FX> constexpr int dslash_min_blocks() {
+    if (P == F64 && !FX) return 0;
     return P == F64 || P == DF32 || (P == F32 && RECON == 18) ? 2 : 3;
 }
+
+// FP64 kernels exist for links as limbs (FX) and, for links that are not unitary and recon 8, for
+// links as doubles with FP64 arithmetic throughout; the launcher chooses by Geom::links_fx.  One
+// kernel with the second form out of line and the layout chosen per load took 2.4 times as long on
+// such links (16^4 256 us against 106, 32^3 x 64 7678 against 3104).  FP64 arithmetic keeps the
+// compiler's choice of registers.
+template <int P, int RECON> constexpr bool fx_form() { return P == F64 && RECON != 8; }
 
 // Site tile (tile_x, in [0, gridDim.x)) and right-hand-side group (tile_y, in
 // [0, gridDim.y)) of this block.  Blocks start in linear order (x fastest); numbering
@@ -1093,8 +1101,8 @@ __device__ __forceinline__ int tile_y() {
 // of site_tile / 2 sites).  Ep::site consumes the hopping sum of one site (or of the
 // lane's two spins); Ep::finish runs once per thread after the loop (block and grid
 // reductions, solver scalars).
-template <int P, int RECON, bool DAG, class Ep, bool EO = false>
-__global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_kernel(DslashArgs a) {
+template <int P, int RECON, bool DAG, class Ep, bool EO = false, bool FX = fx_form<P, RECON>()>
+__global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON, FX>()) dslash_kernel(DslashArgs a) {
     using R = typename Real<P>::T;
     if (a.run_flag && *a.run_flag == 0) return;
     const int r = tile_y() * blockDim.y + threadIdx.y;
@@ -1117,7 +1125,7 @@ __global__ void __launch_bounds__(256, dslash_min_blocks<P, RECON>()) dslash_ker
             const bool on = row && s < a.g.V;
             C<R> own[6];
             // all 32 lanes: row and s0 are the same for them
-            hopping_own<P, RECON, DAG, EO>(a.g, in, a.gauge, a.gauge_dir, s, hh, on && !zin, own);
+            hopping_own<P, RECON, DAG, EO, true, FX>(a.g, in, a.gauge, a.gauge_dir, s, hh, on && !zin, own);
             if (on) Ep::template site<P>(a, s, r, xin, own, st[0], pt);
         }
     } else {

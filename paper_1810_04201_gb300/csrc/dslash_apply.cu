@@ -21,6 +21,12 @@ static cudaError_t go(const DslashArgs &a, DslashTiles t, cudaStream_t st) {
     }
     dim3 block(t.site_tile, t.rhs_tile);
     dim3 grid(site_blocks<P>(a.g.V, t.site_tile), (a.nrhs + t.rhs_tile - 1) / t.rhs_tile);
+    if constexpr (fx_form<P, RECON>()) {
+        if (!a.g.links_fx) {
+            dslash_kernel<P, RECON, DAG, EpXpay, false, false><<<grid, block, 0, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
     dslash_kernel<P, RECON, DAG, EpXpay><<<grid, block, 0, st>>>(a);
     return cudaGetLastError();
 }

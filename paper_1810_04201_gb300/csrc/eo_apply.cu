@@ -9,12 +9,15 @@
 
 using namespace wd;
 
-template <int RECON, bool DAG>
+template <int RECON, bool DAG, bool FX>
 static cudaError_t schur(const DslashArgs &hop, const DslashArgs &back, DslashTiles t, cudaStream_t st) {
+    if constexpr (FX) {
+        if (!hop.g.links_fx) return schur<RECON, DAG, false>(hop, back, t, st);
+    }
     dim3 block(t.site_tile, 1);
     dim3 grid(site_blocks<F64>(hop.g.V, t.site_tile), 1);
-    dslash_kernel<F64, RECON, DAG, EpHop, true><<<grid, block, 0, st>>>(hop);
-    dslash_kernel<F64, RECON, DAG, EpXpay, true><<<grid, block, 0, st>>>(back);
+    dslash_kernel<F64, RECON, DAG, EpHop, true, FX><<<grid, block, 0, st>>>(hop);
+    dslash_kernel<F64, RECON, DAG, EpXpay, true, FX><<<grid, block, 0, st>>>(back);
     return cudaGetLastError();
 }
 
@@ -63,7 +66,8 @@ extern "C" wd_status wd_apply_schur(wd_ctx *c, double kappa, const void *in, voi
     const DslashTiles t = cg_tiles_for(c, F64, 1, true);
     const cudaError_t err = with_recon(link_recon(c, F64), [&](auto rc) {
         constexpr int R = decltype(rc)::value;
-        return dagger ? schur<R, true>(h, b, t, c->stream) : schur<R, false>(h, b, t, c->stream);
+        constexpr bool fx = fx_form<F64, R>();
+        return dagger ? schur<R, true, fx>(h, b, t, c->stream) : schur<R, false, fx>(h, b, t, c->stream);
     });
     WD_CUDA(c, err);
     WD_CUDA(c, cudaMemsetAsync(io, 0, sh, c->stream));

@@ -95,14 +95,18 @@ static inline int num_sms() {
 // tile, left to the hardware scheduler, is slower wherever there are more tiles than that (solves,
 // ms: 24^4 FP32 8.11 against 6.88, FP16 6.62 / 5.69; 20^3 x 40 FP32 with 12 rows 70.4 / 62.2;
 // 16^3 x 32 FP64 9.41 / 8.44), and so are half and twice as many blocks (24^4 FP32 8.62, 7.51).
+// `few` (FP64 arithmetic, where a tile takes long): with at most four tiles per resident block the
+// scheduler does better (solves, one block per tile / resident: 2.7 tiles per block, 16^4 11.7 /
+// 12.7, 16^3 x 32 even-odd 12.0 / 12.6; 5.4 tiles, 16^3 x 32 22.7 / 21.6).
 constexpr int kMaxPartialBlocks = 8192;
 template <int P, class K>
-static dim3 reduce_grid(K kernel, const Geom &g, DslashTiles t, int nrhs, int threads) {
+static dim3 reduce_grid(K kernel, const Geom &g, DslashTiles t, int nrhs, int threads, bool few) {
     const int need = site_blocks<P>(g.V, t.site_tile), rows = (nrhs + t.rhs_tile - 1) / t.rhs_tile;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
     if (per_sm < 1) per_sm = 1;
-    const int cap = per_sm * num_sms() < kMaxPartialBlocks ? per_sm * num_sms() : kMaxPartialBlocks;
+    int cap = per_sm * num_sms() * (few && need <= 4 * per_sm * num_sms() ? 4 : 1);
+    if (cap > kMaxPartialBlocks) cap = kMaxPartialBlocks;
     return dim3(need < cap ? need : cap, rows);
 }
 
@@ -141,12 +145,16 @@ static void add_dslash(GraphBuilder &gb, const DslashArgs &a, DslashTiles t, boo
     const int per = P == F32 && pairs_rows<Ep>() && t.rhs_per_thread == 2 && t.rhs_tile % 2 == 0 ? 2 : 1;
     const dim3 block(t.site_tile, t.rhs_tile / per);
     auto add = [&](auto k) {
-        dim3 grid = reduce ? reduce_grid<P>(k, a.g, t, a.nrhs, block.x * block.y)
+        const bool few = P == F64 && (!fx_form<P, RECON>() || !a.g.links_fx);
+        dim3 grid = reduce ? reduce_grid<P>(k, a.g, t, a.nrhs, block.x * block.y, few)
                            : dim3(site_blocks<P>(a.g.V, t.site_tile), (a.nrhs + t.rhs_tile - 1) / t.rhs_tile);
         gb.kernel(k, grid, block, a);
     };
     if constexpr (P == F32 && pairs_rows<Ep>()) {
         if (per == 2) return add(dslash_multi_kernel<RECON, DAG, 2, Ep, EO>);
+    }
+    if constexpr (fx_form<P, RECON>()) {
+        if (!a.g.links_fx) return add(dslash_kernel<P, RECON, DAG, Ep, EO, false>);
     }
     add(dslash_kernel<P, RECON, DAG, Ep, EO>);
 }

@@ -103,7 +103,7 @@ __global__ void k_face_pack(FaceArgs a) {
     SpinorIO<P>::load(in, a.g.Vs, n1, p);
     project<3, -SF>(p, h);
     C<R> u[9], w[6];
-    load_link<P, RECON>(a.g, reinterpret_cast<const char *>(a.gauge) + 3 * a.gauge_dir, a.g.Vs, n1, u);
+    load_link_of<P, RECON>(a.g, reinterpret_cast<const char *>(a.gauge) + 3 * a.gauge_dir, a.g.Vs, n1, u);
     su3_mult<true>(u, h, w, false);
     FaceIO<P>::store(at_rhs(a.to_next, a.face_stride, r), a.Vfs, f, w);
 }
@@ -134,7 +134,7 @@ __global__ void k_face_apply(FaceArgs a) {
     for (int c = 0; c < 12; ++c) acc1[c] = acc0[c] = C<R>{R(0), R(0)};
     // last slice: forward hop onto the next sub-lattice's first slice
     FaceIO<P>::load(at_rhs(a.from_next, a.face_stride, r), a.Vfs, f, h);
-    load_link<P, RECON>(a.g, reinterpret_cast<const char *>(a.gauge) + 3 * a.gauge_dir, a.g.Vs, n1, u);
+    load_link_of<P, RECON>(a.g, reinterpret_cast<const char *>(a.gauge) + 3 * a.gauge_dir, a.g.Vs, n1, u);
     su3_mult<false>(u, h, w, a.flip_next != 0);
     accumulate<3, SF>(acc1, w);
     // first slice: backward hop from the previous sub-lattice's last slice (U^dag h came with it)

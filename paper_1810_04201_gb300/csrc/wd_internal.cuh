@@ -319,8 +319,9 @@ template <int P, int RECON> struct LinkIO;
 
 template <int RECON> struct LinkIO<F64, RECON> {
     using R = double;
-    // fx: the entries are limbs (recon 18 and 12)
-    static __device__ __forceinline__ void load(const void *dir_base, int Vs, int s, C<R> (&u)[9], bool fx) {
+    // FX: the entries are limbs (recon 18 and 12)
+    template <bool FX>
+    static __device__ __forceinline__ void load(const void *dir_base, int Vs, int s, C<R> (&u)[9]) {
         const double2 *p = reinterpret_cast<const double2 *>(dir_base) + s;
         if constexpr (RECON == 8) {
 #pragma unroll
@@ -335,7 +336,7 @@ template <int RECON> struct LinkIO<F64, RECON> {
         constexpr int n = RECON == 12 ? 6 : 9;
 #pragma unroll
         for (int e = 0; e < n; ++e) {
-            if (fx) {
+            if constexpr (FX) {
                 const int4 t = __ldg(reinterpret_cast<const int4 *>(p) + (size_t)e * Vs);
                 u[e] = C<R>{fx_link_value(t.x, t.y), fx_link_value(t.z, t.w)};
             } else {
@@ -441,12 +442,20 @@ template <int RECON> struct LinkIO<F16, RECON> {
     }
 };
 
-// link of a direction in the layout of the lattice's geometry
-template <int P, int RECON>
-__device__ __forceinline__ void load_link(const Geom &g, const void *dir_base, int Vs, int s,
-                                          C<typename Real<P>::T> (&u)[9]) {
-    if constexpr (P == F64) LinkIO<P, RECON>::load(dir_base, Vs, s, u, g.links_fx != 0);
+// link of a direction; FX: FP64 links as limbs
+template <int P, int RECON, bool FX = false>
+__device__ __forceinline__ void load_link(const void *dir_base, int Vs, int s, C<typename Real<P>::T> (&u)[9]) {
+    if constexpr (P == F64) LinkIO<P, RECON>::template load<FX>(dir_base, Vs, s, u);
     else LinkIO<P, RECON>::load(dir_base, Vs, s, u);
+}
+// the same in the layout of the lattice's geometry
+template <int P, int RECON>
+__device__ __forceinline__ void load_link_of(const Geom &g, const void *dir_base, int Vs, int s,
+                                             C<typename Real<P>::T> (&u)[9]) {
+    if constexpr (P == F64 && RECON != 8) {
+        if (g.links_fx) return load_link<P, RECON, true>(dir_base, Vs, s, u);
+    }
+    load_link<P, RECON>(dir_base, Vs, s, u);
 }
 
 // ------------------------------------------------------------------ reductions

@@ -98,3 +98,57 @@ def test_non_finite_spinors_reach_their_neighbours_only(bad):
     ref = oracle.apply_D(U, clean, KAPPA, DIMS)
     assert not np.isfinite(got[near].reshape(near.sum(), -1)).all(1).any()
     assert oracle.rel_err(got[~near], ref[~near]) < 1e-13
+
+
+def crooked_links(dims, seed):
+    """Haar links with two of them scaled: the FP64 kernels keep such links as doubles."""
+    U = gen.haar_links(dims, seed=seed)
+    U[2, 7] *= 1.2
+    U[0, 3] *= 0.9
+    return U
+
+
+@pytest.mark.parametrize("recon", [18, 12])
+def test_every_fp64_kernel_on_links_that_are_not_unitary(recon):
+    """recon 12 rebuilds row 2 of a scaled link as the square of the scale: its reference has that."""
+    from paper_1810_04201_gb300 import wd
+    dims = (4, 4, 6, 4)
+    U = crooked_links(dims, 3)
+    lat = lattice(U, dims, recon)
+    if recon == 12:
+        U = U.copy()
+        U[..., 2, :] = np.cross(U[..., 0, :], U[..., 1, :]).conj()
+    B = gen.gaussian_source(dims, seed=4, nrhs=2)
+    X = np.stack([oracle.cgnr(U, b, KAPPA, dims, tol=1e-13)[0] for b in B])
+    fb = lat.pack(B)
+    for kw in (dict(), dict(precondition=1), dict(block=1), dict(inner=1), dict(inner=1, precondition=1), dict(normal_eq=1)):
+        fx = lat.new_field(nrhs=2)
+        lat.cg(KAPPA, fb, fx, tol=1e-11, nrhs=2, **kw)
+        assert oracle.rel_err(lat.unpack(fx, nrhs=2), X) < 1e-9, kw
+    fo = lat.new_field()
+    lat.normal_apply_noalloc(KAPPA, lat.pack(B[0]), fo)
+    assert oracle.rel_err(lat.unpack(fo), oracle.apply_normal(U, B[0], KAPPA, dims)) < 1e-13
+    straight = lattice(gen.haar_links(DIMS, seed=5), recon=recon)
+    b5 = gen.gaussian_source(DIMS, seed=6)
+    xs = [lat.new_field(), straight.new_field()]
+    res, st = wd.cg_batched([lat, straight], [KAPPA, KAPPA], [lat.pack(B[0]), straight.pack(b5)], xs, tol=1e-11)
+    assert st == 0
+    assert oracle.rel_err(lat.unpack(xs[0]), X[0]) < 1e-9
+    x5, _ = oracle.cgnr(gen.haar_links(DIMS, seed=5), b5, KAPPA, DIMS, tol=1e-13)
+    assert oracle.rel_err(straight.unpack(xs[1]), x5) < 1e-9
+
+
+def test_fp64_arithmetic_has_its_own_launch_shape():
+    """Where the FP64 units bound the operator (links not unitary, recon 8) blocks stay small."""
+    dims = (16, 16, 32, 32)
+    V = int(np.prod(dims))
+    U = np.tile(gen.haar_links((4, 4, 4, 4), seed=9), (1, V // 256, 1, 1))
+    lat = lattice(U, dims)
+    assert lat.tiles(0, 1) == (256, 1, 1)
+    lat.set_gauge(U, recon=8)
+    assert lat.tiles(0, 1) == (64, 1, 1)
+    U[2, 7] *= 1.2
+    lat.set_gauge(U)
+    assert lat.tiles(0, 1) == (64, 1, 1)
+    lat.set_gauge(U, recon=12)
+    assert lat.tiles(0, 1) == (64, 1, 1)
