@@ -73,10 +73,16 @@ typedef enum wd_status {
 } wd_status;
 
 /* Storage and arithmetic precision of a field and of the operator applied to it.
- *   WD_F64   IEEE double.  For unitary links whole or as recon 12 the products U psi are
- *            formed from integer and FP32 parts relative to the largest neighbouring component
- *            (the operator's relative error is no larger than with IEEE arithmetic); other links,
- *            recon 8 and spinors beyond 2^-894 .. 2^1007 use IEEE arithmetic throughout.
+ *   WD_F64   IEEE double.  For unitary links, whole or as recon 12, the products U psi are
+ *            formed from integer and FP32 parts in units of a power of two at most twice the
+ *            largest component of a site's neighbours: links are held to 2^-56, spinor
+ *            components to 2^-62 and a site's hop sums to some 2^-54 of the unit, absolutely
+ *            and not each relative to itself.  A site with a complex sum below 2^-14 of the
+ *            unit, where a component below 2^-12 of it takes part, is computed with IEEE
+ *            arithmetic (on the links as held); so are sites with spinors beyond
+ *            2^-894 .. 2^1007, other links and recon 8.  In norm, on random SU(3) links and
+ *            Gaussian spinors, the operator's relative error is no larger than with IEEE
+ *            arithmetic (6.2e-17 against 8.2e-17 at kappa = 0.12).
  *   WD_F32   IEEE single.
  *   WD_F16   half-precision storage with a per-site FP32 scale, FP32 accumulation:
  *            the spin projection adds half values in half precision and the SU(3)

@@ -946,9 +946,36 @@ __device__ __noinline__ void half_native(const Geom &g, const void *in, const vo
     hopping_half<F64, RECON, DAG, EO, NC, true>(g, in, gauge, gdir_bytes, s, hh, acc);
 }
 
+// Whether the lane's eight hops read a complex component that is not zero but below
+// 2^-kFxSpreadBits of the unit of exponent E.  Out of line: rarely called.
+template <bool EO, bool NC>
+__device__ __noinline__ bool fx_spread(const Geom &g, const void *in, int s, int hh, int E) {
+    int xc[4], m = s;
+    if constexpr (EO) m = eo_full_index(g, s, xc[0], xc[1], xc[2], xc[3]);
+    else site_xyzt(g, s, xc[0], xc[1], xc[2], xc[3]);
+    bool found = false;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int mu = k >> 1, L = g.L[mu], st = g.stride[mu], c = xc[mu];
+        const bool back = k & 1, edge = c == (back ? 0 : L - 1);
+        if (!EO && mu == 3 && g.split_t && edge) continue;  // left out at a cut
+        const int step = edge ? -(L - 1) * st : st;
+        int n = WD_IDX(g, back ? m - step : m + step, EO ? 2 * g.V : g.V, (EO ? 3 : 1) + back);
+        if (EO) n >>= 1;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            C<double> p[3];
+            load_spin<F64, NC>(in, g.Vs, n, h == 0 ? hh : mu < 2 ? 3 - hh : 2 + hh, p);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) found |= fx_below(p[j].re, p[j].im, E);
+        }
+    }
+    return found;
+}
+
 // The hopping sum of site s for the spins this lane owns (hh and 3 - hh), zero where `on` is
 // false.  Every lane of the warp calls it (on is the same for both lanes of a site).
-// FX: links as limbs (Geom::links_fx), with lanes that the limbs cannot take redone in FP64.
+// FX: links as limbs (Geom::links_fx), with sites that the limbs cannot take redone in FP64.
 template <int P, int RECON, bool DAG, bool EO, bool NC, bool FX>
 __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const void *gauge, size_t gdir_bytes, int s,
                                             int hh, bool on, C<typename Real<P>::T> (&own)[6]) {
@@ -957,7 +984,7 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
         FxAcc acc;
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc.v[k] = 0;
-        acc.E = kFxMinExp;
+        acc.E = kFxMinExp - 1;  // stays there where all spinors are zero
         acc.bad = 0;
         if (on) fx_hopping<RECON, DAG, EO, NC, 1>(g, in, gauge, gdir_bytes, s, hh, acc);
         // both lanes in one unit; the partner's spin 2 + hh' is this lane's 3 - hh
@@ -973,6 +1000,19 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
             own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
         }
         bool native = acc.bad;
+        // Sums far below the unit have few digits left.  That is no loss where large terms cancelled,
+        // but it is where the terms were small, and others, which do not enter this component (links
+        // that do not mix colours, the other spin of a chirality), set the unit.
+        unsigned low = ~0u;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            low = min(low, max((unsigned)((int)(acc.v[2 * k] >> 32) + kFxSmallHi),
+                               (unsigned)((int)(acc.v[2 * k + 1] >> 32) + kFxSmallHi)));
+        bool small = low < 2u * kFxSmallHi && acc.E >= kFxMinExp;
+        if (__any_sync(0xffffffffu, small)) {
+            small |= __shfl_xor_sync(0xffffffffu, small, 16) != 0;  // both lanes' spinors make both lanes' sums
+            if (on && small) native |= fx_spread<EO, NC>(g, in, s, hh, acc.E);
+        }
         if (__any_sync(0xffffffffu, native)) {
             native |= __shfl_xor_sync(0xffffffffu, native, 16) != 0;
             C<double> acc[9];

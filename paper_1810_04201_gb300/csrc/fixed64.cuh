@@ -10,10 +10,12 @@
 //   H H' 2^-60   exact, summed in 64-bit integers, and
 //   (H L' + L H') 2^-92   in FP32,
 // and the sum of the eight hops, an integer in 2^-57 units, becomes a double with one rounding.
-// FP64 arithmetic rounds each partial sum to 2^-53 of itself; the FP32 products are off by 2^-24
-// of 2^-30: the result is closer to the exact operator than with FP64 arithmetic (relative error
-// against 128-bit arithmetic, Haar links, Gaussian spinors: kappa 0.12 8.2e-17 -> 6.2e-17, kappa 1
-// 1.57e-16 -> 1.01e-16, recon-12 at kappa 0.12 1.06e-16 -> 9.1e-17).
+// FP64 arithmetic rounds each partial sum to 2^-53 of itself; here the FP32 products are off by 2^-24
+// of 2^-30 units, spinors by 2^-62 and links by 2^-56.  In norm the result is closer to the exact
+// operator than with FP64 arithmetic (relative error against 128-bit arithmetic, Haar links, Gaussian
+// spinors: kappa 0.12 8.2e-17 -> 6.2e-17, kappa 1 1.57e-16 -> 1.01e-16, recon-12 at kappa 0.12
+// 1.06e-16 -> 9.1e-17).  A component far below the unit is not: what that could lose goes through
+// FP64 arithmetic (kFxSmallBits below).
 // Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 811-850 us (128- and 64-thread blocks),
 // 16^4 107 -> 34.5 us; with recon-12 links 5066 -> 1083 us.  (Three integer products of 29-bit
 // limbs per real product, the first form: 882-888, 36.5 and 1400 us.)  What bounds it now is the
@@ -37,6 +39,13 @@ constexpr float kFxSmallToAcc = 0x1p-35f;        // small products come in units
 // Exponents (biased) of the units this arithmetic takes: below, a scaled result could be
 // subnormal; above, the sum of eight hops could overflow.  Other fields go through FP64.
 constexpr int kFxMinExp = 128, kFxMaxExp = 2030;
+
+// A site with a complex sum whose parts are both below 2^-kFxSmallBits units is redone in FP64 where
+// a complex component that entered its lanes' hops, zeros apart, is below 2^-kFxSpreadBits units
+// (hopping_own).  On Gaussian fields one warp in two million gets as far as looking at the inputs;
+// with the real and imaginary parts each by itself one in a hundred did, and 16^4 took 71 us for 32.
+constexpr int kFxSmallBits = 14, kFxSpreadBits = 12;
+constexpr int kFxSmallHi = 1 << (kFxAccBits - kFxSmallBits - 32);  // that sum's high word
 
 // link entry -> (H, bits of the float L): u = H 2^-30 + L 2^-62
 __device__ __forceinline__ int2 fx_link(double u) {
@@ -83,6 +92,13 @@ __device__ __forceinline__ void fx_sum(double a, int ma, double b, int mb, unsig
     mb ^= __double2hiint(b) >> 31;
     fx_split((long long)(fx_fixed(a, c) ^ (unsigned long long)(long long)ma) +
              (long long)(fx_fixed(b, c) ^ (unsigned long long)(long long)mb) - (ma + mb), h, l);
+}
+
+// re + i im is not zero, but both parts are below 2^-kFxSpreadBits units of exponent E
+__device__ __forceinline__ bool fx_below(double re, double im, int E) {
+    const unsigned long long r = (unsigned long long)__double_as_longlong(re) << 1,
+                             i = (unsigned long long)__double_as_longlong(im) << 1, m = r > i ? r : i;
+    return m != 0 && (int)(m >> 53) <= E - kFxSpreadBits;
 }
 
 __device__ __forceinline__ long long fx_mac(int a, int b, long long s) { return (long long)a * b + s; }

@@ -100,6 +100,60 @@ def test_non_finite_spinors_reach_their_neighbours_only(bad):
     assert oracle.rel_err(got[~near], ref[~near]) < 1e-13
 
 
+@pytest.mark.parametrize("small", [1e-6, 1e-10, 1e-14, 1e-19, 1e-120])
+@pytest.mark.parametrize("recon", [18, 12])
+def test_colours_far_below_the_others_keep_their_digits(small, recon):
+    """Unit links do not mix colours, so every colour is right to its own rounding: what falls below
+    2^-14 of the lane's unit is computed with IEEE arithmetic."""
+    U = gen.unit_links(DIMS)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    psi[:, :, 1] *= small
+    psi[:, :, 2] *= small ** 2 if small > 1e-100 else 0.0
+    lat = lattice(U, recon=recon)
+    for dagger in (False, True):
+        got, ref = apply(lat, psi, dagger), oracle.apply_D(U, psi, KAPPA, DIMS, dagger=dagger)
+        for c in range(3):
+            assert np.linalg.norm(got[:, :, c] - ref[:, :, c]) <= 1e-15 * np.linalg.norm(ref[:, :, c])
+
+
+@pytest.mark.parametrize("spin", range(4))
+def test_spins_far_below_the_others_keep_their_digits(spin):
+    """The hops into a spin never read the other spin of its chirality, but its lane takes its unit from
+    that one too: with only that one large, the spin keeps its own digits."""
+    U = gen.haar_links(DIMS, seed=3)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    psi[:, spin] *= 1e10
+    lat = lattice(U)
+    for dagger in (False, True):
+        got = apply(lat, psi, dagger)[:, spin ^ 1]
+        ref = oracle.apply_D(U, psi, KAPPA, DIMS, dagger=dagger)[:, spin ^ 1]
+        assert np.linalg.norm(got - ref) <= 1e-15 * np.linalg.norm(ref)
+
+
+def test_components_above_the_limit_are_within_the_stated_bound():
+    """Colours 1e-4 and 1e-2 of the largest on unit links.  A hop is off by at most 2^-56 of the unit
+    for its low limb's 24 bits and 2^-57 for the rounding of its sums, eight hops by 24 x 2^-57, and the
+    unit is at most twice the largest component of the neighbourhood."""
+    U = gen.unit_links(DIMS)
+    psi = gen.gaussian_source(DIMS, seed=4)
+    psi[:, :, 1] *= 1e-4
+    psi[:, :, 2] *= 1e-2
+    err = np.abs(apply(lattice(U), psi) - oracle.apply_D(U, psi, KAPPA, DIMS))[:, :, 1].reshape(len(psi), -1).max(1)
+    assert np.all(err <= 24 * 2.0 ** -56 * KAPPA * neighbourhood_max(psi, DIMS))
+
+
+@pytest.mark.parametrize("dims", [DIMS, (16, 8, 8, 8)])
+def test_sparse_fields_are_exact_zeros_and_right(dims):
+    """One colour of one spin on unit links: most sums are zeros, which are looked at again."""
+    U = gen.unit_links(dims)
+    psi = gen.gaussian_source(dims, seed=4)
+    psi[:, :, 1:] = 0
+    psi[:, 1:] = 0
+    got, ref = apply(lattice(U, dims), psi), oracle.apply_D(U, psi, KAPPA, dims)
+    assert np.all(got[ref == 0] == 0)
+    assert oracle.rel_err(got, ref) < 1e-15
+
+
 def crooked_links(dims, seed):
     """Haar links with two of them scaled: the FP64 kernels keep such links as doubles."""
     U = gen.haar_links(dims, seed=seed)
