@@ -773,24 +773,8 @@ __device__ __forceinline__ void fx_load_link(const char *gdir, int Vs, int s, in
     constexpr int n = RECON == 12 ? 6 : 9;
 #pragma unroll
     for (int e = 0; e < n; ++e) u[e] = __ldg(p + (size_t)e * Vs);
-    if constexpr (RECON == 12) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            // conj(a b - c d) with a = u[i], b = u[3 + j], c = u[j], d = u[3 + i]
-            const int i = (k + 1) % 3, j = (k + 2) % 3;
-            const int4 a = u[i], b = u[3 + j], c = u[j], d = u[3 + i];
-            long long hr = 0, hi = 0;
-            float fr = 0.f, fi = 0.f;
-            fx_cmac<false>(a, b.x, -b.z, b.z, b.x, (float)b.x, (float)b.z, __int_as_float(b.y), __int_as_float(b.w), hr, hi, fr, fi);
-            long long gr = 0, gi = 0;
-            float er = 0.f, ei = 0.f;
-            fx_cmac<false>(c, d.x, -d.z, d.z, d.x, (float)d.x, (float)d.z, __int_as_float(d.y), __int_as_float(d.w), gr, gi, er, ei);
-            const int2 re = fx_link_of(hr - gr, fr - er), im = fx_link_of(gi - hi, ei - fi);
-            u[6 + k] = make_int4(re.x, re.y, im.x, im.y);
-        }
-    }
+    if constexpr (RECON == 12) fx_row2(u);
 }
-
 
 // the sums in the larger unit of exponent e
 __device__ __forceinline__ void fx_raise(FxAcc &acc, int e) {

@@ -23,12 +23,14 @@
 // add and FP64 pipes are busy 47, 39 and 38 % of the cycles, DRAM 32 %, issue slots 50 %.
 //
 // Bounds.  A spinor component is a sum of two doubles, each below (1 - 2^-21) units, so H fits 32
-// bits; |L| <= 2^31; links |H| <= 2^30 (1 + 2^-11) with rows and columns of norm at most
-// 1 + 2^-10.  By Cauchy and Schwarz a sum of six products H H' is below sqrt(6) 2^61 (1 + 2^-10)
-// < 2^62.3, the small ones, in units of the sums, below 2^30, one hop below sqrt(6) 2^58 and
-// eight hops below 2^62.3.
+// bits; |L| <= 2^31 (a rebuilt row's 2^31 + 2^10); links |H| <= 2^30 (1 + 2^-11) with rows and columns of
+// norm at most 1 + 2^-10.  By Cauchy and Schwarz a sum of six products H H' is below sqrt(6) 2^61
+// (1 + 2^-10) < 2^62.3, the small ones, in units of the sums, below 2^30, one hop below sqrt(6) 2^58
+// and eight hops below 2^62.3.
 #pragma once
 #include <cuda_runtime.h>
+#include <cmath>
+#include <cstring>
 
 namespace wd {
 
@@ -47,13 +49,33 @@ constexpr int kFxMinExp = 128, kFxMaxExp = 2030;
 constexpr int kFxSmallBits = 14, kFxSpreadBits = 12;
 constexpr int kFxSmallHi = 1 << (kFxAccBits - kFxSmallBits - 32);  // that sum's high word
 
-// link entry -> (H, bits of the float L): u = H 2^-30 + L 2^-62
-__device__ __forceinline__ int2 fx_link(double u) {
-    const int h = __double2int_rn(u * kFxLinkScale);
-    return make_int2(h, __float_as_int((float)(fma((double)h, -0x1p-30, u) * 0x1p62)));
+// a float of given bits and a float's bits, on either side (the arithmetic of a link is also compiled
+// for the host, where tests look at the limbs)
+__host__ __device__ __forceinline__ float fx_float(int b) {
+#ifdef __CUDA_ARCH__
+    return __int_as_float(b);
+#else
+    float f;
+    memcpy(&f, &b, sizeof f);
+    return f;
+#endif
 }
-__device__ __forceinline__ double fx_link_value(int h, int l) {
-    return fma((double)h, 0x1p-30, (double)__int_as_float(l) * 0x1p-62);
+__host__ __device__ __forceinline__ int fx_bits(float f) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(f);
+#else
+    int b;
+    memcpy(&b, &f, sizeof b);
+    return b;
+#endif
+}
+// link entry -> (H, bits of the float L): u = H 2^-30 + L 2^-62
+__host__ __device__ __forceinline__ int2 fx_link(double u) {
+    const int h = (int)rint(u * kFxLinkScale);
+    return make_int2(h, fx_bits((float)(fma((double)h, -0x1p-30, u) * 0x1p62)));
+}
+__host__ __device__ __forceinline__ double fx_link_value(int h, int l) {
+    return fma((double)h, 0x1p-30, (double)fx_float(l) * 0x1p-62);
 }
 
 // the larger of m and the |hi words| of two doubles, as float bits; NaN for words from
@@ -101,28 +123,51 @@ __device__ __forceinline__ bool fx_below(double re, double im, int E) {
     return m != 0 && (int)(m >> 53) <= E - kFxSpreadBits;
 }
 
-__device__ __forceinline__ long long fx_mac(int a, int b, long long s) { return (long long)a * b + s; }
+__host__ __device__ __forceinline__ long long fx_mac(int a, int b, long long s) { return (long long)a * b + s; }
 
 // (hr, hi, fr, fi) += u z (ADJ: conj(u) z) for a link entry u and z = x + iy with limbs
 // (x, xf = float(x), xl) and likewise y; mre, mim: the factors of u's imaginary limb in the
 // real and the imaginary part (ADJ ? y : -y, ADJ ? -x : x).  hr, hi: exact products of the high
 // limbs; fr, fi: the cross products in FP32, in units 2^-32 of those.
 template <bool ADJ>
-__device__ __forceinline__ void fx_cmac(int4 u, int x, int mre, int y, int mim, float xf, float yf, float xl, float yl,
+__host__ __device__ __forceinline__ void fx_cmac(int4 u, int x, int mre, int y, int mim, float xf, float yf, float xl, float yl,
                                         long long &hr, long long &hi, float &fr, float &fi) {
-    const float rf = (float)u.x, rl = __int_as_float(u.y), jf = ADJ ? -(float)u.z : (float)u.z,
-                jl = ADJ ? -__int_as_float(u.w) : __int_as_float(u.w);
+    const float rf = (float)u.x, rl = fx_float(u.y), jf = ADJ ? -(float)u.z : (float)u.z,
+                jl = ADJ ? -fx_float(u.w) : fx_float(u.w);
     hr = fx_mac(u.z, mre, fx_mac(u.x, x, hr));
     hi = fx_mac(u.z, mim, fx_mac(u.x, y, hi));
     fr = fmaf(-jl, yf, fmaf(-jf, yl, fmaf(rl, xf, fmaf(rf, xl, fr))));
     fi = fmaf(jl, xf, fmaf(jf, xl, fmaf(rl, yf, fmaf(rf, yl, fi))));
 }
 
-// The link entry of the value h 2^-60 + f 2^-92
-__device__ __forceinline__ int2 fx_link_of(long long h, float f) {
+// The link entry of the value h 2^-60 + f 2^-92.  The cross sums f of a rebuilt entry (up to 2^63)
+// take L past 2^31 several times over; what is over is carried to H, so that |L| <= 2^31 + 2^10, as of
+// a stored entry but for rounding.  Rounded by a magic addition: conversions of f to an integer and
+// back cost 2 % of a recon-12 operator.
+__host__ __device__ __forceinline__ int2 fx_link_of(long long h, float f) {
+    constexpr float magic = 0x1.8p23f;
     const int q = (int)((h + (1ll << 29)) >> 30);
     const int r = (int)(h - ((long long)q << 30));
-    return make_int2(q, __float_as_int(fmaf((float)r, 4.f, f * 0x1p-30f)));
+    const float l = fmaf((float)r, 4.f, f * 0x1p-30f), m = fmaf(l, 0x1p-32f, magic);
+    return make_int2(q + (fx_bits(m) - fx_bits(magic)), fx_bits(fmaf(m - magic, -0x1p32f, l)));
+}
+
+// Row 2 = conj(row0 x row1) of a recon-12 link in the same arithmetic.
+__host__ __device__ __forceinline__ void fx_row2(int4 (&u)[9]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        // conj(a b - c d) with a = u[i], b = u[3 + j], c = u[j], d = u[3 + i]
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        const int4 a = u[i], b = u[3 + j], c = u[j], d = u[3 + i];
+        long long hr = 0, hi = 0;
+        float fr = 0.f, fi = 0.f;
+        fx_cmac<false>(a, b.x, -b.z, b.z, b.x, (float)b.x, (float)b.z, fx_float(b.y), fx_float(b.w), hr, hi, fr, fi);
+        long long gr = 0, gi = 0;
+        float er = 0.f, ei = 0.f;
+        fx_cmac<false>(c, d.x, -d.z, d.z, d.x, (float)d.x, (float)d.z, fx_float(d.y), fx_float(d.w), gr, gi, er, ei);
+        const int2 re = fx_link_of(hr - gr, fr - er), im = fx_link_of(gi - hi, ei - fi);
+        u[6 + k] = make_int4(re.x, re.y, im.x, im.y);
+    }
 }
 
 // v 2^e as a double, rounded once; e = (exponent of the unit) - 1022 - kFxAccBits
