@@ -180,19 +180,19 @@ __device__ void for_tiles_half(const BatchArgs &a, W &&want, F &&body) {
 // with the partner lane: the lane's two spins (SiteHalf).  Every lane of the warp
 // calls it.  Plain loads: the fields change between the phases of one launch.  Out of line:
 // seven inlined copies would not fit the instruction cache.  A batch may hold lattices with links
-// as limbs and others with links as doubles (FX = false).
-template <int RECON, bool DAG, bool FX>
-__device__ __noinline__ void hop64_form(const LatDesc &L, const void *in, int s, int hh, bool on,
-                                        C<double> (&own)[6]) {
-    hopping_own<F64, RECON, DAG, false, false, FX>(L.g, in, L.g64, L.gdir64, s, hh, on, own);
+// as limbs and others with links as doubles, whose form is a function of its own.
+template <int RECON, bool DAG>
+__device__ __noinline__ void hop64_native(const LatDesc &L, const void *in, int s, int hh, bool on,
+                                          C<double> (&own)[6]) {
+    hopping_own<F64, RECON, DAG, false, false, false>(L.g, in, L.g64, L.gdir64, s, hh, on, own);
 }
 template <int RECON, bool DAG>
-__device__ __forceinline__ void hop64_half(const LatDesc &L, const void *in, int s, int hh, bool on,
-                                           C<double> (&own)[6]) {
+__device__ __noinline__ void hop64_half(const LatDesc &L, const void *in, int s, int hh, bool on,
+                                        C<double> (&own)[6]) {
     if constexpr (fx_form<F64, RECON>()) {
-        if (L.g.links_fx) return hop64_form<RECON, DAG, true>(L, in, s, hh, on, own);
+        if (!L.g.links_fx) return hop64_native<RECON, DAG>(L, in, s, hh, on, own);
     }
-    hop64_form<RECON, DAG, false>(L, in, s, hh, on, own);
+    hopping_own<F64, RECON, DAG, false, false, fx_form<F64, RECON>()>(L.g, in, L.g64, L.gdir64, s, hh, on, own);
 }
 
 // kBlocksPerSm blocks of 128 threads per SM (96 registers): the inner FP32 phases, which wait on

@@ -983,7 +983,6 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
             own[k] = C<R>{fx_value(acc.v[2 * k], e), fx_value(acc.v[2 * k + 1], e)};
             own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
         }
-        bool native = acc.bad;
         // Sums far below the unit have few digits left.  That is no loss where large terms cancelled,
         // but it is where the terms were small, and others, which do not enter this component (links
         // that do not mix colours, the other spin of a chirality), set the unit.
@@ -992,21 +991,21 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
         for (int k = 0; k < 6; ++k)
             low = min(low, max((unsigned)((int)(acc.v[2 * k] >> 32) + kFxSmallHi),
                                (unsigned)((int)(acc.v[2 * k + 1] >> 32) + kFxSmallHi)));
-        bool small = low < 2u * kFxSmallHi && acc.E >= kFxMinExp;
-        if (__any_sync(0xffffffffu, small)) {
+        bool small = low < 2u * kFxSmallHi && acc.E >= kFxMinExp, native = acc.bad;
+        if (__any_sync(0xffffffffu, small || native)) {
             small |= __shfl_xor_sync(0xffffffffu, small, 16) != 0;  // both lanes' spinors make both lanes' sums
             if (on && small) native |= fx_spread<EO, NC>(g, in, s, hh, acc.E);
-        }
-        if (__any_sync(0xffffffffu, native)) {
             native |= __shfl_xor_sync(0xffffffffu, native, 16) != 0;
-            C<double> acc[9];
+            if (__any_sync(0xffffffffu, native)) {
+                C<double> acc9[9];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) acc[k] = C<double>{0.0, 0.0};
-            if (on && native) half_native<RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc);
-            exchange_halves(acc);
-            if (native)
+                for (int k = 0; k < 9; ++k) acc9[k] = C<double>{0.0, 0.0};
+                if (on && native) half_native<RECON, DAG, EO, NC>(g, in, gauge, gdir_bytes, s, hh, acc9);
+                exchange_halves(acc9);
+                if (native)
 #pragma unroll
-                for (int k = 0; k < 6; ++k) own[k] = acc[k];
+                    for (int k = 0; k < 6; ++k) own[k] = acc9[k];
+            }
         }
     } else {
         C<R> acc[9];
