@@ -264,9 +264,8 @@ typedef struct wd_cg_params {
 
 /* Per right-hand side result.  The two residuals are recomputed from the returned x
  * with the FP64 operator: by a final check after the loop, or, where a mixed-precision
- * solve (or a batched lattice) stopped at a reliable update, by that update, which
- * computed D x and D^dag(b - D x) for the same x (even-odd: the even half of b - D x, the
- * odd half vanishes but for rounding since x_o = b_o + kappa H_oe x_e). */
+ * solve on the full lattice (or a batched lattice) stopped at a reliable update, by
+ * that update, which computed D x and D^dag(b - D x) for the same x. */
 typedef struct wd_cg_result {
     int iters;               /* CG iterations */
     int reliable_updates;    /* FP64 residual recomputations (mixed precision) */

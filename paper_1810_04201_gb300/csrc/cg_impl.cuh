@@ -138,25 +138,16 @@ static void record_plan(wd_ctx *c, const SolverPlan &pl, const Fields &f, const 
                 DslashArgs r = base;
                 r.mask = 2;
                 r.in = f.x; r.out = f.t;
-                if constexpr (EO) {
-                    // the reduced residual t = b^ - S x and r = S^dag t, with the norms of the
-                    // full-lattice residuals: an update that stops a row is its final check
+                if constexpr (!EO && !NE) {
+                    // t = D x with |b - t|^2: an update that stops a row is its final check
                     r.a0 = f.b;
-                    add_op<F64, RECON, OP1, EpResid, EO>(ib, r, pl.t64, true, f);
-                    r.in = f.t; r.a0 = nullptr; r.a1 = f.r;
-                    add_op<F64, RECON, OP2, EpReliable<true>, EO, EpHopNorm>(ib, r, pl.t64, true, f);
+                    add_op<F64, RECON, OP1, EpTrue1, EO>(ib, r, pl.t64, true, f);
+                    r.a0 = nullptr;
                 } else {
-                    if constexpr (!NE) {
-                        // t = D x with |b - t|^2: an update that stops a row is its final check
-                        r.a0 = f.b;
-                        add_op<F64, RECON, OP1, EpTrue1, EO>(ib, r, pl.t64, true, f);
-                        r.a0 = nullptr;
-                    } else {
-                        add_op<F64, RECON, OP1, EpXpay, EO>(ib, r, pl.t64, false, f);
-                    }
-                    r.in = f.t; r.a0 = f.db; r.a1 = f.r;
-                    add_op<F64, RECON, OP2, EpReliable<false>, EO>(ib, r, pl.t64, true, f);
+                    add_op<F64, RECON, OP1, EpXpay, EO>(ib, r, pl.t64, false, f);
                 }
+                r.in = f.t; r.a0 = f.db; r.a1 = f.r;
+                add_op<F64, RECON, OP2, EpReliable, EO>(ib, r, pl.t64, true, f);
                 v.a = f.r; v.a_stride = s64; v.b = f.rs; v.b_stride = sin;
                 add_vec(ib, k_convert<F64, SP>, v);
                 if constexpr (SP == F16) {
@@ -231,9 +222,9 @@ static void record_plan(wd_ctx *c, const SolverPlan &pl, const Fields &f, const 
         dbt = f.p;
     }
     a.in = xf; a.out = tf; a.a0 = bf;
-    // mixed precision (CGNR): skipped when every row stopped at a reliable update, which
-    // computed these norms for the x it returns (state[4] = 0)
-    if (mixed && !NE) a.run_flag = f.state + 4;
+    // mixed precision on the full lattice: skipped when every row stopped at a reliable
+    // update, which computed these norms for the x it returns (state[4] = 0)
+    if (mixed && !EO && !NE) a.run_flag = f.state + 4;
     add_dslash<F64, RECON, false, EpTrue1>(gb, a, pl.t64, true);
     a.in = tf; a.a0 = dbt;
     add_dslash<F64, RECON, true, EpTrue2>(gb, a, pl.t64, true);

@@ -248,51 +248,7 @@ struct EpCG2Mixed {
     }
 };
 
-// Even-odd reliable update, pass 1: the residual of the reduced system, out = b^ - S x (b^ = a0)
-// and |out|^2 -> true_b2.  With x_o = b_o + kappa H_oe x_e this is the even half of b - D x, and
-// the odd half vanishes, so the update knows the full-lattice residuals too: |b - D x| = |out| and
-// |D^dag (b - D x)|^2 = |out|^2 + kappa^2 |H_oe^dag out|^2, the second from the bare hop of pass 2.
-struct EpResid {
-    struct State { double v[1]; };
-    template <int P, class R, class Pt>
-    static __device__ __forceinline__ void site(const DslashArgs &a, int s, int r, const void *in, C<R> (&acc)[Pt::N],
-                                                State &st, const Pt &pt) {
-        C<R> p[Pt::N], b[Pt::N];
-        load_part<P>(pt, in, a.g.Vs, s, p);
-        xpay_site(p, acc, R(a.kappa));
-        load_part<P>(pt, rhs_ptr<R>(a.a0, a.a0_stride, r), a.g.Vs, s, b);
-#pragma unroll
-        for (int c = 0; c < Pt::N; ++c) b[c] = csub(b[c], p[c]);
-        st.v[0] += norm2_of(b);
-        store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, b);
-    }
-    template <int P, int K>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
-        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].true_b2 = t[0]; });
-    }
-};
-
-// Pass 2's bare hop: out = -kappa * hop, |out|^2 -> odd2
-struct EpHopNorm {
-    struct State { double v[1]; };
-    template <int P, class R, class Pt>
-    static __device__ __forceinline__ void site(const DslashArgs &a, int s, int r, const void *, C<R> (&acc)[Pt::N],
-                                                State &st, const Pt &pt) {
-        const R k = R(-a.kappa);
-#pragma unroll
-        for (int c = 0; c < Pt::N; ++c) acc[c] = C<R>{k * acc[c].re, k * acc[c].im};
-        st.v[0] += norm2_of(acc);
-        store_part<P>(pt, rhs_ptr<R>(a.out, a.out_stride, r), a.g.Vs, s, acc);
-    }
-    template <int P, int K>
-    static __device__ __forceinline__ void finish(const DslashArgs &a, int r, State (&st)[K]) {
-        reduce_finish<1>(a, r, st, [&](int row, const double *t) { a.sc[row].odd2 = t[0]; });
-    }
-};
-
-// Reliable update, FP64: q = D^dag t (t = D x); r = db - q (a1, db = a0); rho = |r|^2.
-// EO: t = b^ - S x (EpResid), r = S^dag t.
-template <bool EO>
+// Reliable update, FP64: q = D^dag t (t = D x); r = db - q (a1, db = a0); rho = |r|^2
 struct EpReliable {
     struct State { double v[1]; };
     template <int P, class R, class Pt>
@@ -301,9 +257,9 @@ struct EpReliable {
         C<R> q[Pt::N], d[Pt::N];
         load_part<P>(pt, in, a.g.Vs, s, q);
         xpay_site(q, acc, R(a.kappa));
-        if constexpr (!EO) load_part<P>(pt, rhs_ptr<R>(a.a0, a.a0_stride, r), a.g.Vs, s, d);
+        load_part<P>(pt, rhs_ptr<R>(a.a0, a.a0_stride, r), a.g.Vs, s, d);
 #pragma unroll
-        for (int c = 0; c < Pt::N; ++c) d[c] = EO ? q[c] : csub(d[c], q[c]);
+        for (int c = 0; c < Pt::N; ++c) d[c] = csub(d[c], q[c]);
         st.v[0] += norm2_of(d);
         store_part<P>(pt, rhs_ptr<R>(a.a1, a.a1_stride, r), a.g.Vs, s, d);
     }
@@ -324,7 +280,7 @@ struct EpReliable {
                 // this update checked the x the row returns: state[3] counts such rows, and
                 // state[4] (the final check's run flag where a plan allows) drops to 0
                 // once every row has stopped this way
-                c.true_n2 = EO ? c.true_b2 + a.kappa * c.odd2 : rt;  // EO: the kernel's kappa is kappa^2
+                c.true_n2 = rt;
                 a.state[3] += 1;
                 a.state[4] = a.state[3] < a.nrhs;
             }

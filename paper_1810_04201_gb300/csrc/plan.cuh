@@ -177,9 +177,9 @@ struct SolverPlan {
 
 // One application of the solver's operator: D (or D^dag) on the full lattice, or,
 // with even-odd preconditioning, the Schur operator 1 - kappa^2 H_eo H_oe (or its
-// adjoint) as two checkerboard kernels: a bare hop (HopEp) into an odd temporary, then
+// adjoint) as two checkerboard kernels: a bare hop into an odd temporary, then
 // the hop back with the epilogue, which adds the even input.
-template <int P, int RECON, bool DAG, class Ep, bool EO, class HopEp = EpHop>
+template <int P, int RECON, bool DAG, class Ep, bool EO>
 static void add_op(GraphBuilder &gb, const DslashArgs &a, DslashTiles t, bool reduce, const Fields &f) {
     if constexpr (!EO) {
         add_dslash<P, RECON, DAG, Ep>(gb, a, t, reduce);
@@ -196,7 +196,7 @@ static void add_op(GraphBuilder &gb, const DslashArgs &a, DslashTiles t, bool re
         h.xsrc = nullptr;
         // a zero input (in_nonzero flag 0) needs no bare hop: the epilogue kernel skips it too
         if (a.in_nonzero) h.run_flag = a.in_nonzero, h.in_nonzero = nullptr;
-        add_dslash<P, RECON, DAG, HopEp, true>(gb, h, t, !std::is_same_v<HopEp, EpHop>);
+        add_dslash<P, RECON, DAG, EpHop, true>(gb, h, t, false);
         DslashArgs e = a;
         e.g = f.eo.ge;
         e.gauge = f.eo.gauge[P];

@@ -564,7 +564,6 @@ struct Scalars {
     double rmax2_lo;   // max |r|^2 since the last correction or reliable update
     int do_correct;    // FP32 correction requested for this iteration
     int corrections;   // FP32 corrections run
-    double odd2;       // even-odd: |H_oe^dag r|^2 of the reduced residual r (last reliable update)
 };
 
 __device__ __forceinline__ bool row_on(const Scalars *sc, int mask, int r) {

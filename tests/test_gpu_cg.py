@@ -663,3 +663,27 @@ def test_rows_in_pairs_match_single_rows(wd, nrhs, eo):
         assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
         out.append(fx.view(torch.float64).clone())
     assert float((out[0] - out[1]).norm() / out[1].norm()) < 2e-9
+
+
+@pytest.mark.parametrize("inner", [1, 2, 3])
+def test_even_odd_residuals_include_the_odd_half(wd, inner):
+    """The reported residuals are those of the returned x on the whole lattice.  With a source on
+    the odd sites just below one and a tiny kappa, x_o = b_o + kappa H_oe x_e rounds by up to 2^-53
+    where it passes one, so b - D x is some 5e-17 |b| on the odd sites, while the even ones, solved in
+    units of kappa, are exact to 1e-20 |b|: a residual of the even sites alone would miss it."""
+    dims, kappa = (4, 4, 6, 8), 1e-5
+    U = gen.haar_links(dims, seed=11)
+    x, y, z, t = np.meshgrid(*[np.arange(n) for n in dims], indexing="ij")
+    odd = ((x + y + z + t) & 1).transpose(3, 2, 1, 0).reshape(-1).astype(bool)
+    g = gen.gaussian_source(dims, seed=12)
+    b = np.where(odd[:, None, None], np.copysign(1 - 2.0 ** -53, g.real) + 1j * np.copysign(1 - 2.0 ** -53, g.imag), 0)
+    lat = wd.Lattice(dims)
+    lat.set_gauge(U)
+    fx = lat.new_field()
+    res, st = lat.cg(kappa, lat.pack(b), fx, tol=1e-12, inner=inner, precondition=1)
+    assert st == 0
+    r = b - oracle.apply_D(U, lat.unpack(fx), kappa, dims)
+    want = np.linalg.norm(r) / np.linalg.norm(b)
+    assert want > 1e-17  # the rounding described above
+    assert 0.3 * want < res[0]["true_rel_resid_b"] < 3 * want
+    assert 0.3 * want < res[0]["true_rel_resid"] < 3 * want
