@@ -118,7 +118,8 @@ wd_status wd_set_stream(wd_ctx *ctx, void *stream);
  * in section 6.1; SU(3) links with |U01|^2 + |U02|^2 >= 1e-6 on every link, so not the
  * unit gauge: otherwise WD_ERR_ARG, and the context holds no gauge field until the
  * next successful call).  The lower-precision copies used by WD_F32/WD_F16/WD_DF32
- * operators are derived from the same field when first needed. */
+ * operators are derived from the same field when first needed after it, though not
+ * inside a stream capture (WD_ERR_STATE: one such call outside the capture makes them). */
 wd_status wd_set_gauge(wd_ctx *ctx, const double *U_canon, int on_device, int recon);
 
 /* Debug builds (libwd compiled with -DWD_DEBUG; the library's tests build one in

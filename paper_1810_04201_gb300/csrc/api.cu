@@ -65,11 +65,25 @@ static wd_status link_buffer(wd_ctx *c, void **buf, int *have, int recon, size_t
     return WD_OK;
 }
 
+// A copy of the links is not made inside a stream capture: it would only be filled when the graph
+// runs, while this context took it as filled for every call from now on.
+static wd_status not_capturing(wd_ctx *c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(c->stream, &st);
+    if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) return WD_OK;
+    if (e != cudaSuccess && e != cudaErrorStreamCaptureImplicit) return cuda_fail(c, e, "cudaStreamIsCapturing");
+    cudaGetLastError();
+    return fail(c, WD_ERR_STATE, "the links have no copy for this call yet, and none is made inside a stream capture: "
+                                 "one such call outside it first");
+}
+
 wd_status gauge_get(wd_ctx *c, Prec p, const void **out) {
     if (!c->has_gauge) return fail(c, WD_ERR_STATE, "no gauge field set (call wd_set_gauge first)");
     if (!c->gauge_ok[p]) {
-        wd_status s = link_buffer(c, &c->gauge[p], &c->gauge_recon[p], link_recon(c, p),
-                                  gauge_bytes(p, link_recon(c, p), c->g.Vs));
+        wd_status s = not_capturing(c);
+        if (s != WD_OK) return s;
+        s = link_buffer(c, &c->gauge[p], &c->gauge_recon[p], link_recon(c, p),
+                        gauge_bytes(p, link_recon(c, p), c->g.Vs));
         if (s != WD_OK) return s;
         void *d = c->gauge[p];
         const size_t dir = gauge_dir_bytes(c, p);
@@ -153,7 +167,9 @@ wd_status gauge_get_eo(wd_ctx *c, Prec p, const void **out, size_t *dir_bytes) {
     const int Vhs = eo_geom(c, 0).Vs;
     const size_t dir = round_up(link_dir_bytes(p, link_recon(c, p), Vhs), 256);
     if (!c->gauge_eo_ok[p]) {
-        wd_status s = link_buffer(c, &c->gauge_eo[p], &c->gauge_eo_recon[p], link_recon(c, p), 8 * dir);
+        wd_status s = not_capturing(c);
+        if (s != WD_OK) return s;
+        s = link_buffer(c, &c->gauge_eo[p], &c->gauge_eo_recon[p], link_recon(c, p), 8 * dir);
         if (s != WD_OK) return s;
         void *d = c->gauge_eo[p];
         with_recon(link_recon(c, p), [&](auto rc) {

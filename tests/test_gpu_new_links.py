@@ -81,3 +81,38 @@ def test_new_links_wait_for_operators_on_an_earlier_stream(on_device):
             lat.apply(KAPPA, f, lat.new_field(prec), prec)
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+def test_links_are_not_converted_inside_a_stream_capture():
+    """A copy of the links that a capture would have to make is refused, as it always was for one
+    that had to be allocated: it would only be filled when the graph runs."""
+    import torch
+    from paper_1810_04201_gb300 import wd
+    U1, U2 = gen.haar_links(DIMS, seed=1), gen.haar_links(DIMS, seed=2)
+    src = gen.gaussian_source(DIMS, seed=3)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        lat = wd.Lattice(DIMS)
+        lat.set_gauge(U1)
+        f, out = lat.pack(src, 1), lat.new_field(1)
+        lat.apply(KAPPA, f, out, 1)
+        lat.set_gauge(U2)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=torch.cuda.current_stream()):
+            out.zero_()
+            with pytest.raises(wd.WDError) as e:
+                lat.apply(KAPPA, f, out, 1)
+        assert e.value.status == 8
+        lat.apply(KAPPA, f, out, 1)
+        fresh = wd.Lattice(DIMS)
+        fresh.set_gauge(U2)
+        want = fresh.new_field(1)
+        fresh.apply(KAPPA, f, want, 1)
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        graph = torch.cuda.CUDAGraph()  # with the copy in place the operator is captured
+        with torch.cuda.graph(graph, stream=torch.cuda.current_stream()):
+            lat.apply(KAPPA, f, out, 1)
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
