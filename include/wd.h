@@ -38,7 +38,8 @@
  *
  * Ownership and streams.  The caller owns every field and canonical buffer; the
  * context owns its gauge copies, its workspace and its CUDA graphs, and frees
- * them in wd_destroy.  Every call is asynchronous on the context's stream, except
+ * them in wd_destroy (gauge copies that new links have not refilled also before it
+ * allocates anything else).  Every call is asynchronous on the context's stream, except
  * the solvers, which wait for the result to fill wd_cg_result, the calls
  * whose on_device flag is 0 (host buffers), which return once the host buffer
  * may be reused, and wd_set_gauge, which waits for earlier work and for its check

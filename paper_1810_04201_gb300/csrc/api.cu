@@ -20,6 +20,40 @@ wd_status cuda_fail(wd_ctx *c, cudaError_t e, const char *where) {
     return fail(c, e == cudaErrorMemoryAllocation ? WD_ERR_OOM : WD_ERR_CUDA, m);
 }
 
+// A copy of the links is not made inside a stream capture: it would only be filled when the graph
+// runs, while this context took it as filled for every call from now on.
+static wd_status not_capturing(wd_ctx *c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(c->stream, &st);
+    if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) return WD_OK;
+    if (e != cudaSuccess && e != cudaErrorStreamCaptureImplicit) return cuda_fail(c, e, "cudaStreamIsCapturing");
+    cudaGetLastError();
+    return fail(c, WD_ERR_STATE, "the links have no copy for this call yet, and none is made inside a stream capture: "
+                                 "one such call outside it first");
+}
+
+// Frees the link copies that new links or another compression left to be refilled (wd_ctx.h) and that
+// have not been, with the graphs that hold their addresses: called before device memory is allocated,
+// so that a context never holds more than its present use and what it last held for refilling.
+static void free_stale_copies(wd_ctx *c) {
+    bool any = false;
+    for (int p = 0; p < kNumPrec; ++p)
+        any |= (c->gauge[p] && !c->gauge_ok[p]) || (c->gauge_eo[p] && !c->gauge_eo_ok[p]);
+    if (!any || not_capturing(c) != WD_OK) return;
+    cudaStreamSynchronize(c->stream);
+    for (int p = 0; p < kNumPrec; ++p) {
+        if (c->gauge[p] && !c->gauge_ok[p]) {
+            cudaFree(c->gauge[p]);
+            c->gauge[p] = nullptr;
+        }
+        if (c->gauge_eo[p] && !c->gauge_eo_ok[p]) {
+            cudaFree(c->gauge_eo[p]);
+            c->gauge_eo[p] = nullptr;
+        }
+    }
+    graph_clear(c);
+}
+
 wd_status ws_get(wd_ctx *c, const std::string &name, size_t bytes, void **out) {
     auto it = c->ws.find(name);
     if (it != c->ws.end() && c->ws_size[name] >= bytes) {
@@ -33,6 +67,7 @@ wd_status ws_get(wd_ctx *c, const std::string &name, size_t bytes, void **out) {
         // graphs may hold the old pointer
         graph_clear(c);
     }
+    free_stale_copies(c);
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) return cuda_fail(c, e, ("cudaMalloc(" + name + ")").c_str());
@@ -51,30 +86,13 @@ static void gauge_pack(const double *canon, void *dst, const Geom &g, size_t dir
 }
 
 // *buf: a device buffer for links of compression recon (its size depends on that alone); one of
-// another compression is freed, with the graphs that hold its address
+// another compression, stale by then, is freed
 static wd_status link_buffer(wd_ctx *c, void **buf, int *have, int recon, size_t bytes) {
     if (*buf && *have == recon) return WD_OK;
-    if (*buf) {
-        WD_CUDA(c, cudaStreamSynchronize(c->stream));
-        cudaFree(*buf);
-        *buf = nullptr;
-        graph_clear(c);
-    }
+    free_stale_copies(c);
     WD_CUDA(c, cudaMalloc(buf, bytes));
     *have = recon;
     return WD_OK;
-}
-
-// A copy of the links is not made inside a stream capture: it would only be filled when the graph
-// runs, while this context took it as filled for every call from now on.
-static wd_status not_capturing(wd_ctx *c) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    const cudaError_t e = cudaStreamIsCapturing(c->stream, &st);
-    if (e == cudaSuccess && st == cudaStreamCaptureStatusNone) return WD_OK;
-    if (e != cudaSuccess && e != cudaErrorStreamCaptureImplicit) return cuda_fail(c, e, "cudaStreamIsCapturing");
-    cudaGetLastError();
-    return fail(c, WD_ERR_STATE, "the links have no copy for this call yet, and none is made inside a stream capture: "
-                                 "one such call outside it first");
 }
 
 wd_status gauge_get(wd_ctx *c, Prec p, const void **out) {

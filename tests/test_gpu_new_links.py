@@ -116,3 +116,30 @@ def test_links_are_not_converted_inside_a_stream_capture():
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(out, want)
+
+
+def test_link_copies_that_the_new_configuration_does_not_use_are_given_back():
+    """A configuration that works in another precision holds what a new context would: the copies
+    kept for refilling go before others are allocated."""
+    import torch
+    from paper_1810_04201_gb300 import wd
+    dims = (16, 16, 16, 16)  # a DF32 copy of the links is 38 MB
+    U = torch.from_numpy(gen.haar_links((4, 4, 4, 4), seed=1)).cuda().repeat(1, 256, 1, 1).contiguous()
+
+    def held(precs):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        lat = wd.Lattice(dims)
+        for prec in precs:
+            lat.set_gauge(U)
+            lat.apply(KAPPA, src[prec], dst[prec], prec)
+        torch.cuda.synchronize()
+        n = free - torch.cuda.mem_get_info()[0]
+        lat.close()
+        return n
+
+    one = wd.Lattice(dims)
+    src, dst = [one.new_field(p) for p in range(4)], [one.new_field(p) for p in range(4)]
+    held([1])
+    assert held([3, 1]) <= held([1]) + (4 << 20)
+    assert held([3, 2, 1, 2]) <= held([1]) + (4 << 20)
