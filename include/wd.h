@@ -312,8 +312,9 @@ wd_status wd_cg_solve_batched(wd_ctx *const *ctxs, const double *kappas, const v
  * the fastest for later calls.  Writes the choice to *site_tile and *rhs_tile
  * (either may be NULL).  Uses context-owned scratch fields; synchronises the stream. */
 wd_status wd_autotune(wd_ctx *ctx, wd_prec prec, int nrhs, int *site_tile, int *rhs_tile);
-/* Autotuner of the solvers: times the same candidates for the fused CG kernels (the
- * Dslash with the CG epilogues and reductions) as wd_cg_solve runs them -- ten iterations
+/* Autotuner of the solvers: times the same candidates (FP32: with one and with two right-hand
+ * sides per thread) for the fused CG kernels (the Dslash with the CG epilogues and reductions) as
+ * wd_cg_solve runs them -- ten iterations
  * of the device-resident loop in inner precision prec (WD_F64: the plain FP64 solver) on a
  * non-zero right-hand side, L2 flushed before each timed solve -- and keeps the fastest
  * for the solvers of this precision and nrhs (wd_cg_solve, wd_cg_solve_canonical); with all
@@ -427,13 +428,17 @@ wd_status wd_measure_fp64_rate(double *gflops);
 /* The launch shape the plain operators of (prec, nrhs) use now: site_tile, rhs_tile and
  * rhs_per_thread (any pointer may be NULL). */
 wd_status wd_get_tiles(wd_ctx *ctx, wd_prec prec, int nrhs, int *site_tile, int *rhs_tile, int *rhs_per_thread);
+/* The same for the fused kernels of wd_cg_solve in inner precision prec (WD_F64: also the FP64
+ * kernels of every solve), plain or even-odd; params.rhs_tile overrides it. */
+wd_status wd_get_cg_tiles(wd_ctx *ctx, wd_prec prec, int nrhs, int precondition, int *site_tile, int *rhs_tile,
+                          int *rhs_per_thread);
 /* Plain FP32 operators: each thread applies its site's links to k (1 to 4) of its block's
  * right-hand sides, loading each link once for all k (k dividing rhs_tile, and
  * site_tile * rhs_tile / k threads a multiple of 32); wd_autotune considers k = 2, 3, 4
  * beside 1.  Other precisions, the solvers' fused kernels and split sub-lattices
- * (WD_ERR_STATE for k > 1): k = 1 only.  (The FP32 solver kernels choose by themselves
- * whether a thread takes one or two right-hand sides.)  No counterpart in the paper, which
- * has one right-hand side. */
+ * (WD_ERR_STATE for k > 1): k = 1 only.  (The FP32 solver kernels take one or two per thread:
+ * as wd_autotune_cg found, else by a rule of their own, on any shape that allows it.)  No
+ * counterpart in the paper, which has one right-hand side. */
 wd_status wd_set_rhs_per_thread(wd_ctx *ctx, wd_prec prec, int nrhs, int k);
 
 /* Launch-configuration query: number of kernel launches the last wd_* call queued

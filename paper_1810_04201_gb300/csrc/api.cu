@@ -249,27 +249,30 @@ void graph_clear(wd_ctx *c) {
 // 29.0); single rows below keep 64 (128: -7 to +3 %, by how the last wave fills).
 // With FP64 arithmetic (fx_links) 64 x 1 everywhere (64 x 1 / 64 x 4 / 256 x 1, four rows: 8^3 x 12 5.77 /
 // 7.39 / 7.28, 16^3 x 32 82.1 / 84.3 / 81.5, even-odd 43.3 / 44.5 / 44.4).
+static bool rows_in_pairs(wd_ctx *c, Prec p, int nrhs, bool eo) {
+    return p == F32 && link_recon(c, p) != 8 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) &&
+           (long long)(c->g.V / (eo ? 2 : 1)) * nrhs >= (1 << 17);
+}
+
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
     auto it = c->cg_tiles.find(p * 64 + nrhs + (eo ? kEoTileKey : 0));
     if (it != c->cg_tiles.end()) return it->second;
     it = c->tiles.find(p * 64 + nrhs);
     DslashTiles t;
     if (it != c->tiles.end()) {
-        t = it->second;
-        t.rhs_per_thread = 1;  // chosen for the plain operators
-        return t;
+        t = it->second;  // chosen for the plain operators, as are its right-hand sides per thread
+    } else {
+        t.site_tile = 64;
+        t.rhs_tile = nrhs < 4 ? nrhs : 4;
+        const long long sites = c->g.V / (eo ? 2 : 1);
+        if (p == F64 && !fx_links(c)) {
+            t.rhs_tile = 1;
+        } else if (p == F64 && (nrhs > 1 || sites >= (1 << 17))) {
+            t.site_tile = sites >= (1 << 17) ? 256 : 128;
+            t.rhs_tile = 1;
+        }
     }
-    t.site_tile = 64;
-    t.rhs_tile = nrhs < 4 ? nrhs : 4;
-    const long long sites = c->g.V / (eo ? 2 : 1), work = sites * nrhs;
-    if (p == F64 && !fx_links(c)) {
-        t.rhs_tile = 1;
-    } else if (p == F64 && (nrhs > 1 || sites >= (1 << 17))) {
-        t.site_tile = sites >= (1 << 17) ? 256 : 128;
-        t.rhs_tile = 1;
-    }
-    if (p == F32 && link_recon(c, p) != 8 && nrhs % 2 == 0 && (nrhs == 4 || (eo && nrhs > 4)) && work >= (1 << 17))
-        t.rhs_per_thread = 2;
+    t.rhs_per_thread = rows_in_pairs(c, p, nrhs, eo) && pairs_fit(t) ? 2 : 1;
     return t;
 }
 

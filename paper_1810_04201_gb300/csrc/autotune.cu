@@ -125,12 +125,24 @@ wd_status wd_get_tiles(wd_ctx *c, wd_prec prec, int nrhs, int *site_tile, int *r
     return WD_OK;
 }
 
+wd_status wd_get_cg_tiles(wd_ctx *c, wd_prec prec, int nrhs, int precondition, int *site_tile, int *rhs_tile,
+                          int *rhs_per_thread) {
+    if (!c || (int)prec < 0 || (int)prec >= kNumPrec || nrhs < 1 || nrhs > WD_MAX_RHS ||
+        (precondition != WD_PRECOND_NONE && precondition != WD_PRECOND_EO))
+        return WD_ERR_ARG;
+    const DslashTiles t = cg_tiles_for(c, (Prec)prec, nrhs, precondition == WD_PRECOND_EO);
+    if (site_tile) *site_tile = t.site_tile;
+    if (rhs_tile) *rhs_tile = t.rhs_tile;
+    if (rhs_per_thread) *rhs_per_thread = t.rhs_per_thread;
+    return WD_OK;
+}
+
 wd_status wd_set_rhs_per_thread(wd_ctx *c, wd_prec prec, int nrhs, int k) {
     if (!c) return WD_ERR_ARG;
     if ((int)prec < 0 || (int)prec >= kNumPrec || nrhs < 1 || nrhs > WD_MAX_RHS || k < 1 || k > 4)
         return fail(c, WD_ERR_ARG, "wd_set_rhs_per_thread: bad argument");
     DslashTiles t = tiles_for(c, (Prec)prec, nrhs);
-    if (!c->tiles.count((int)prec * 64 + nrhs)) {  // no shape chosen yet: k of up to four rows of a block
+    if (k > 1 && !c->tiles.count((int)prec * 64 + nrhs)) {  // no shape chosen yet: k of up to four rows of a block
         t.site_tile = 64;
         t.rhs_tile = nrhs < 4 ? nrhs : 4;
     }

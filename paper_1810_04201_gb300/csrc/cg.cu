@@ -320,7 +320,8 @@ wd_status wd_cg_solve_canonical(wd_ctx *c, double kappa, const double *b_canon, 
 
 // Solver autotuner: the launch shape of the fused CG kernels is timed as the solver runs
 // them, a fixed number of iterations of the device-resident loop on a non-zero right-hand
-// side, with L2 flushed before each timed solve (the candidates as in wd_autotune).
+// side, with L2 flushed before each timed solve (the candidates as in wd_autotune, FP32 with one
+// and two right-hand sides per thread; the default shape is among them).
 wd_status wd_autotune_cg(wd_ctx *c, wd_prec prec, int nrhs, int *site_tile, int *rhs_tile) {
     wd::NvtxRange nvtx_("wd_autotune_cg");
     if (!c) return WD_ERR_ARG;
@@ -358,30 +359,33 @@ wd_status wd_autotune_cg(wd_ctx *c, wd_prec prec, int nrhs, int *site_tile, int 
         double best = 1e30;
         DslashTiles bt = cg_tiles_for(c, (Prec)prec, nrhs, pc != 0);
         for (int st : sts)
-            for (int rt : rts) {
-                if (rt > nrhs || st * rt > 256 || (st * rt) % 32 != 0) continue;
-                if (threads_per_site((Prec)prec) > 1 && st % 32 != 0) continue;
-                DslashTiles t;
-                t.site_tile = st;
-                t.rhs_tile = rt;
-                c->cg_tiles[key] = t;
-                double secs = 0.0;
-                for (int rep = 0; rep < 2; ++rep) {  // the first run builds and uploads the graph
-                    WD_CUDA(c, cudaMemsetAsync(x, 0, fb, c->stream));
-                    WD_CUDA(c, cudaMemsetAsync(flush, rep, flush_bytes, c->stream));
-                    s = wd_cg_solve(c, 0.12, b, x, &prm, res.data());
-                    if (s != WD_OK && s != WD_ERR_NOT_CONVERGED) {
-                        c->cg_tiles[key] = bt;
-                        return s;
+            for (int rt : rts)
+                for (int kt = 1; kt <= (prec == WD_F32 ? 2 : 1); ++kt) {
+                    if (rt > nrhs || st * rt > 256 || (st * rt) % 32 != 0) continue;
+                    if (threads_per_site((Prec)prec) > 1 && st % 32 != 0) continue;
+                    DslashTiles t;
+                    t.site_tile = st;
+                    t.rhs_tile = rt;
+                    t.rhs_per_thread = kt;
+                    if (kt == 2 && !pairs_fit(t)) continue;
+                    c->cg_tiles[key] = t;
+                    double secs = 0.0;
+                    for (int rep = 0; rep < 2; ++rep) {  // the first run builds and uploads the graph
+                        WD_CUDA(c, cudaMemsetAsync(x, 0, fb, c->stream));
+                        WD_CUDA(c, cudaMemsetAsync(flush, rep, flush_bytes, c->stream));
+                        s = wd_cg_solve(c, 0.12, b, x, &prm, res.data());
+                        if (s != WD_OK && s != WD_ERR_NOT_CONVERGED) {
+                            c->cg_tiles[key] = bt;
+                            return s;
+                        }
+                        launches += c->launches;
+                        secs = res[0].seconds;
                     }
-                    launches += c->launches;
-                    secs = res[0].seconds;
+                    if (secs < best) {
+                        best = secs;
+                        bt = t;
+                    }
                 }
-                if (secs < best) {
-                    best = secs;
-                    bt = t;
-                }
-            }
         c->cg_tiles[key] = bt;
         if (pc == 0) chosen = bt;
     }

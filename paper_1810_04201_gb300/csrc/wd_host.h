@@ -107,6 +107,8 @@ DslashTiles tiles_for(wd_ctx *c, Prec p, int nrhs);
 // wd_autotune_cg's choice, else the one chosen for the plain operators, else the default
 constexpr int kEoTileKey = 1024;
 DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo);
+// whether a block of this shape can take its rows in pairs, two right-hand sides per thread
+inline bool pairs_fit(const DslashTiles &t) { return t.rhs_tile % 2 == 0 && t.site_tile * t.rhs_tile / 2 % 32 == 0; }
 // frees a workspace buffer (no-op when absent)
 void ws_release(wd_ctx *c, const std::string &name);
 

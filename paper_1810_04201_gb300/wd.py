@@ -94,6 +94,7 @@ def load_library(path: str = LIB_PATH):
         "wd_autotune_cg": ([P, I, I, ctypes.POINTER(I), ctypes.POINTER(I)], I),
         "wd_set_staging": ([P, I, I, I], I),
         "wd_get_tiles": ([P, I, I, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I)], I),
+        "wd_get_cg_tiles": ([P, I, I, I, ctypes.POINTER(I), ctypes.POINTER(I), ctypes.POINTER(I)], I),
         "wd_set_rhs_per_thread": ([P, I, I, I], I),
         "wd_staging_error": ([P, ctypes.POINTER(ctypes.c_uint)], I),
         "wd_set_prefetch": ([P, I, I], I),
@@ -315,6 +316,13 @@ class Lattice:
         a, b, k = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         self._check(self.lib.wd_get_tiles(self.ctx, prec, nrhs, ctypes.byref(a), ctypes.byref(b), ctypes.byref(k)),
                     "wd_get_tiles")
+        return a.value, b.value, k.value
+
+    def cg_tiles(self, prec=WD_F64, nrhs=1, precondition=0):
+        """(site_tile, rhs_tile, rhs_per_thread) the solver's kernels of inner precision prec use."""
+        a, b, k = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+        self._check(self.lib.wd_get_cg_tiles(self.ctx, prec, nrhs, precondition, ctypes.byref(a), ctypes.byref(b),
+                                             ctypes.byref(k)), "wd_get_cg_tiles")
         return a.value, b.value, k.value
 
     def set_rhs_per_thread(self, prec, nrhs, k):

@@ -637,32 +637,101 @@ def test_even_odd_reports_the_residuals_of_what_it_returns(wd, inner, nrhs, tol,
         assert (res[k]["status"] == 0) == (want_n <= tol)
 
 
-@pytest.mark.parametrize("nrhs,eo", [(4, 0), (4, 1), (6, 1), (12, 1)])
-def test_rows_in_pairs_match_single_rows(wd, nrhs, eo):
+def solve_with_rhs_tile(wd, lat, kappa, fb, fx, nrhs, eo, rhs_tile, tol=1e-10):
+    """An FP32 mixed solve with params.rhs_tile, which also fixes one right-hand side per thread."""
+    import ctypes
+    p = lat.params(tol=tol, nrhs=nrhs, rhs_tile=rhs_tile, inner=1, precondition=eo)
+    res = (wd.CGResult * nrhs)()
+    st = lat.lib.wd_cg_solve(lat.ctx, kappa, ctypes.c_void_p(fb.data_ptr()), ctypes.c_void_p(fx.data_ptr()),
+                             ctypes.byref(p), res)
+    return [r.as_dict() for r in res], st
+
+
+@pytest.mark.parametrize("recon_in", [18, 12])
+@pytest.mark.parametrize("nrhs,eo,dims", [(4, 0, (16, 16, 16, 16)), (4, 0, (15, 17, 13, 11)), (4, 1, (16, 16, 16, 32)),
+                                          (6, 1, (16, 16, 16, 16)), (12, 1, (14, 10, 18, 10))])
+def test_rows_in_pairs_match_single_rows(wd, nrhs, eo, dims, recon_in):
     """From 2^17 site-rows on the FP32 iteration takes two right-hand sides per thread: the same
-    arithmetic, so the solutions agree with those of one row per thread but for the order of the sums
-    over sites, which moves alpha and beta by a few 1e-16 (FP32 rounding of the iterates: 1e-7 of a
-    residual that the FP64 updates then correct, so both meet 1e-10; 16 sites of tile keep one row)."""
-    dims, kappa = (16, 16, 16, 16 if eo == 0 or nrhs > 4 else 32), 0.12
+    arithmetic, so the iterations and solutions agree with those of one row per thread but for the
+    order of the sums over sites, which moves alpha and beta by a few 1e-16 (FP32 rounding of the
+    iterates: 1e-7 of a residual that the FP64 updates then correct, so both meet 1e-10).  Site
+    counts that no tile divides; row 1 of its pair starts from its solution and is left out early."""
     import torch
+    kappa = 0.12
     g = torch.Generator(device="cuda").manual_seed(7)
-    U = gen.haar_links((4, 4, 4, 4), seed=5)
     V = int(np.prod(dims))
-    Ug = torch.from_numpy(U).cuda().reshape(4, 256, 9).repeat(1, V // 256, 1).reshape(4, V, 3, 3).contiguous()
+    U = torch.from_numpy(gen.haar_links((4, 4, 4, 4), seed=5)).cuda()
+    U = torch.stack([U[mu][torch.randint(256, (V,), generator=g, device="cuda")] for mu in range(4)])
     B = torch.complex(torch.randn(nrhs, V, 4, 3, generator=g, device="cuda", dtype=torch.float64),
                       torch.randn(nrhs, V, 4, 3, generator=g, device="cuda", dtype=torch.float64))
     lat = wd.Lattice(dims)
-    lat.set_gauge(Ug)
+    lat.set_gauge(U)
+    if recon_in != 18:
+        lat.set_link_compression(1, recon_in)
+    assert lat.cg_tiles(1, nrhs, eo) == (64, 4, 2)
     fb = lat.pack(B)
-    out = []
-    for paired in (True, False):
-        if not paired:
-            lat.set_tiles(1, nrhs, 64, 2)
+    out, its = [], []
+    for rhs_tile in (0, 2, 0):
         fx = lat.new_field(nrhs=nrhs)
-        res, st = lat.cg(kappa, fb, fx, tol=1e-10, inner=1, nrhs=nrhs, precondition=eo)
+        if out:
+            fx.view(nrhs, -1)[1].copy_(out[0].view(torch.uint8).view(nrhs, -1)[1])
+        res, st = solve_with_rhs_tile(wd, lat, kappa, fb, fx, nrhs, eo, rhs_tile)
         assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
         out.append(fx.view(torch.float64).clone())
-    assert float((out[0] - out[1]).norm() / out[1].norm()) < 2e-9
+        its.append([r["iters"] for r in res])
+    assert its[1][1] == its[2][1] == 0 and min(its[1][:1] + its[1][2:]) > 10
+    for k in (1, 2):
+        assert all(abs(a - b) <= 1 for a, b in zip(its[1], its[2]))
+        assert float((out[k] - out[0]).norm() / out[0].norm()) < 2e-9
+
+
+def test_pairs_survive_a_shape_chosen_for_the_plain_operators(wd):
+    """wd_set_tiles and wd_autotune choose for the plain operators; the solver keeps their block
+    shape, and its own rule for pairs where the shape allows them."""
+    dims = (16, 16, 16, 16)
+    lat = wd.Lattice(dims)
+    lat.set_gauge(np.tile(gen.haar_links((4, 4, 4, 4), seed=5), (1, 256, 1, 1)))
+    assert lat.cg_tiles(1, 4) == (64, 4, 2)
+    lat.set_tiles(1, 4, 64, 2)
+    assert lat.cg_tiles(1, 4) == (64, 2, 2) and lat.tiles(1, 4) == (64, 2, 1)
+    lat.set_tiles(1, 4, 64, 1)
+    assert lat.cg_tiles(1, 4) == (64, 1, 1)
+    lat.set_tiles(1, 4, 16, 2)
+    assert lat.cg_tiles(1, 4) == (16, 2, 1)  # 16 threads are no warp
+    lat.set_tiles(1, 2, 64, 2)
+    assert lat.cg_tiles(1, 2) == (64, 2, 1)  # two rows gain nothing
+    st_, rt = lat.autotune(1, 4)
+    assert lat.cg_tiles(1, 4)[:2] == (st_, rt) and lat.cg_tiles(1, 4)[2] == (2 if rt % 2 == 0 else 1)
+
+
+def test_autotune_cg_times_every_shape_with_pairs(wd):
+    """Two solves of ten iterations per candidate, plain and even-odd, pairs among them: counted by
+    their launches, which do not depend on the shape."""
+    lat = wd.Lattice((4, 4, 4, 8))
+    lat.set_gauge(gen.haar_links((4, 4, 4, 8), seed=83))
+    nrhs = 4
+    per = []
+    for eo in (0, 1):
+        fx = lat.new_field(nrhs=nrhs)
+        lat.cg(0.12, lat.pack(gen.gaussian_source((4, 4, 4, 8), seed=84, nrhs=nrhs)), fx, tol=1e-20, max_iter=10, inner=1,
+               nrhs=nrhs, precondition=eo, raise_on_fail=False)
+        per.append(lat.launches)
+    shapes = [(s, r) for s in (16, 32, 64, 128, 256) for r in (1, 2, 3, 4) if s * r <= 256 and s * r % 32 == 0]
+    n = len(shapes) + sum(r % 2 == 0 and s * r // 2 % 32 == 0 for s, r in shapes)
+    lat.autotune_cg(1, nrhs)
+    assert lat.launches == 1 + 2 * n * sum(per)
+    assert lat.cg_tiles(1, nrhs)[2] in (1, 2)
+
+
+def test_one_right_hand_side_per_thread_keeps_the_default_shape(wd):
+    """wd_set_rhs_per_thread with k = 1 changes no block shape, tuned or not."""
+    dims = (16, 16, 16, 16)
+    lat = wd.Lattice(dims)
+    lat.set_gauge(np.tile(gen.haar_links((4, 4, 4, 4), seed=5), (1, 256, 1, 1)))
+    for prec, nrhs in ((0, 12), (0, 1), (1, 4), (1, 3), (2, 12), (3, 2)):
+        before = lat.tiles(prec, nrhs)
+        lat.set_rhs_per_thread(prec, nrhs, 1)
+        assert lat.tiles(prec, nrhs) == before[:2] + (1,)
 
 
 @pytest.mark.parametrize("inner", [1, 2, 3])
