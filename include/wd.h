@@ -437,7 +437,7 @@ wd_status wd_get_cg_tiles(wd_ctx *ctx, wd_prec prec, int nrhs, int precondition,
  * site_tile * rhs_tile / k threads a multiple of 32); wd_autotune considers k = 2, 3, 4
  * beside 1.  Other precisions, the solvers' fused kernels and split sub-lattices
  * (WD_ERR_STATE for k > 1): k = 1 only.  (The FP32 solver kernels take one or two per thread:
- * as wd_autotune_cg found, else by a rule of their own, on any shape that allows it.)  No
+ * as wd_autotune_cg found, else by a rule of their own.)  No
  * counterpart in the paper, which has one right-hand side. */
 wd_status wd_set_rhs_per_thread(wd_ctx *ctx, wd_prec prec, int nrhs, int k);
 

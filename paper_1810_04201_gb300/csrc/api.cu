@@ -239,9 +239,14 @@ void graph_clear(wd_ctx *c) {
 // sides per block (12 rows of FP32 at 24^3 x 48: 128.9 ms a solve against 129.8 with one and
 // 130.8 with two per block; the plain operators differ, see tiles_for).  FP32 rows go in pairs on
 // one thread from 2^17 site-rows on with four rows (24^3 x 48: 41.3 -> 39.6 ms) and, even-odd, with
-// more (20^3 x 40, 12 rows 37.9 -> 36.3); two rows gain nothing (21.2 / 21.7 ms), and 12 rows on the
-// whole lattice lose (126 / 134 ms).  With recon-12 links the pairs still gain (four rows at
+// more (20^3 x 40, 12 rows 37.9 -> 36.3); two rows gain nothing (21.2 / 21.7 ms).  More rows on the
+// whole lattice gain on small ones and lose on large ones, and stay single (single / pairs, ms a
+// solve: 16^3 x 32 six rows 15.0 / 13.6, eight 17.3 / 16.3, sixteen 33.5 / 31.7; 24^3 x 48 six
+// 64.6 / 66.2, eight 77.2 / 81.3, ten 102.9 / 109.3, twelve 116.9 / 125.6; recon-12 eight rows 15.8 /
+// 16.0 and 75.5 / 79.3).  With recon-12 links the pairs of the rule still gain (four rows at
 // 16^3 x 32 even-odd 6.13 -> 5.65 ms, at 24^4 19.6 -> 19.1), with recon-8 they lose (24^3 x 48 37.5 / 40.0).
+// On a shape chosen for the plain operators they need its four rows: with two per block, four rows of
+// 24^3 x 48 take 40.3 ms in pairs and 40.0 singly, of 16^3 x 32 9.51 and 9.21.
 // FP64 takes one row per block, which shares links through L2 as well and wastes no lanes: blocks of
 // 256 threads from 2^17 sites on (64 / 256, ms a solve: 16^3 x 32 24.8 / 23.0, 24^3 x 48 113.9 / 105.1,
 // even-odd 39.5 / 38.3, 12 rows 1255 (64 x 4) / 1237), 128 below with several rows (64 x 4 / 128 x 1,
@@ -272,7 +277,7 @@ DslashTiles cg_tiles_for(wd_ctx *c, Prec p, int nrhs, bool eo) {
             t.rhs_tile = 1;
         }
     }
-    t.rhs_per_thread = rows_in_pairs(c, p, nrhs, eo) && pairs_fit(t) ? 2 : 1;
+    t.rhs_per_thread = rows_in_pairs(c, p, nrhs, eo) && t.rhs_tile >= 4 && pairs_fit(t) ? 2 : 1;
     return t;
 }
 

@@ -687,21 +687,18 @@ def test_rows_in_pairs_match_single_rows(wd, nrhs, eo, dims, recon_in):
 
 def test_pairs_survive_a_shape_chosen_for_the_plain_operators(wd):
     """wd_set_tiles and wd_autotune choose for the plain operators; the solver keeps their block
-    shape, and its own rule for pairs where the shape allows them."""
+    shape, and its own rule for pairs where a block has four rows or more."""
     dims = (16, 16, 16, 16)
     lat = wd.Lattice(dims)
     lat.set_gauge(np.tile(gen.haar_links((4, 4, 4, 4), seed=5), (1, 256, 1, 1)))
     assert lat.cg_tiles(1, 4) == (64, 4, 2)
-    lat.set_tiles(1, 4, 64, 2)
-    assert lat.cg_tiles(1, 4) == (64, 2, 2) and lat.tiles(1, 4) == (64, 2, 1)
-    lat.set_tiles(1, 4, 64, 1)
-    assert lat.cg_tiles(1, 4) == (64, 1, 1)
-    lat.set_tiles(1, 4, 16, 2)
-    assert lat.cg_tiles(1, 4) == (16, 2, 1)  # 16 threads are no warp
+    for shape, k in (((64, 4), 2), ((32, 4), 2), ((64, 2), 1), ((64, 1), 1), ((16, 2), 1)):
+        lat.set_tiles(1, 4, *shape)
+        assert lat.cg_tiles(1, 4) == shape + (k,) and lat.tiles(1, 4) == shape + (1,)
     lat.set_tiles(1, 2, 64, 2)
     assert lat.cg_tiles(1, 2) == (64, 2, 1)  # two rows gain nothing
     st_, rt = lat.autotune(1, 4)
-    assert lat.cg_tiles(1, 4)[:2] == (st_, rt) and lat.cg_tiles(1, 4)[2] == (2 if rt % 2 == 0 else 1)
+    assert lat.cg_tiles(1, 4) == (st_, rt, 2 if rt == 4 else 1)
 
 
 def test_autotune_cg_times_every_shape_with_pairs(wd):
