@@ -195,29 +195,61 @@ def test_batched_full_c5_workload(wd, rin):
     assert len({r["iters"] for r in res}) > 1
 
 
-def test_a_batch_large_enough_for_two_sites_per_thread(wd):
-    """From 4 x 256 x the resident blocks sites on a tile holds two sites per thread; volumes that
-    are no multiple of a tile, against the same lattices solved alone."""
+@pytest.mark.parametrize("inner,recon_in,start", [(1, 18, False), (1, 18, True), (1, 12, False), (2, 18, True), (2, 12, False)])
+def test_a_batch_large_enough_for_two_sites_per_thread(wd, inner, recon_in, start):
+    """From 4 x 256 sites for each of five resident blocks per SM on a tile holds two sites per thread
+    (a quarter more than that here, on whatever GPU runs it); volumes that are no multiple of a tile,
+    and start vectors on some lattices, against the same lattices solved alone."""
     import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    count = int(1.25 * 4 * 256 * 5 * sms / 16 ** 4) + 1
     g = torch.Generator(device="cuda").manual_seed(3)
-    small = gen.haar_links((4, 4, 4, 4), seed=9)
-    shapes = [(16, 16, 16, 16)] * 12 + [(15, 13, 7, 5), (6, 5, 7, 9)]
+    small = torch.from_numpy(gen.haar_links((4, 4, 4, 4), seed=9)).cuda()
+    shapes = [(16, 16, 16, 16)] * count + [(15, 13, 7, 5), (6, 5, 7, 9)]
     lats, bs, xs = [], [], []
     for dims in shapes:
         V = int(np.prod(dims))
-        idx = torch.randint(256, (4, V), generator=g, device="cuda")
-        U = torch.from_numpy(small).cuda()
-        U = torch.stack([U[mu][idx[mu]] for mu in range(4)])
+        U = torch.stack([small[mu][torch.randint(256, (V,), generator=g, device="cuda")] for mu in range(4)])
         b = torch.complex(*[torch.randn(V, 4, 3, generator=g, device="cuda", dtype=torch.float64) for _ in range(2)])
         lat = wd.Lattice(dims)
         lat.set_gauge(U)
+        if recon_in != 18:
+            lat.set_link_compression(inner, recon_in)
         lats.append(lat)
         bs.append(lat.pack(b))
-        xs.append(lat.new_field())
+        xs.append(lat.pack(0.1 * b) if start and len(xs) % 2 else lat.new_field())
     kappas = [0.11] * len(shapes)
-    res, st = wd.cg_batched(lats, kappas, bs, xs, tol=1e-10, inner=1)
+    res, st = wd.cg_batched(lats, kappas, bs, xs, tol=1e-10, inner=inner)
     assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
-    for i in (0, 11, 12, 13):
+    for i in (0, 1, count - 1, count, count + 1):
         x1 = lats[i].new_field()
-        lats[i].cg(kappas[i], bs[i], x1, tol=1e-10, inner=1)
+        lats[i].cg(kappas[i], bs[i], x1, tol=1e-10, inner=inner)
         assert oracle.rel_err(lats[i].unpack(xs[i]), lats[i].unpack(x1)) < 1e-9
+
+
+@pytest.mark.parametrize("inner", [1, 2])
+def test_fields_of_very_different_magnitude_in_one_batch(wd, inner):
+    """The FP64 phases on sources of 1e-12 and 1e12, on sites that differ by six decades, on unit
+    links that keep colours apart (one of them 1e-8 of the others) and on links that are not unitary,
+    all in one launch, against the oracle."""
+    dims = (4, 4, 6, 8)
+    U = gen.haar_links(dims, seed=3)
+    bent = U.copy()
+    bent[1, 5] *= 1.1
+    b = gen.gaussian_source(dims, seed=4)
+    spread = b * (10.0 ** (6 * gen.uniform(5, gen.STREAM_MISC, 0, len(b)) - 3))[:, None, None]
+    faint = b.copy()
+    faint[:, :, 2] *= 1e-8
+    items = [(U, b * 1e-12), (U, b * 1e12), (U, spread), (gen.unit_links(dims), faint), (bent, b), (bent, spread)]
+    lats, bs, xs = [], [], []
+    for u, src in items:
+        lats.append(wd.Lattice(dims))
+        lats[-1].set_gauge(u)
+        bs.append(lats[-1].pack(src))
+        xs.append(lats[-1].new_field())
+    res, st = wd.cg_batched(lats, [0.11] * len(items), bs, xs, tol=1e-10, inner=inner)
+    assert st == 0 and all(r["true_rel_resid"] <= 1e-10 for r in res)
+    for lat, x, (u, src) in zip(lats, xs, items):
+        scale = np.abs(src).max()
+        want, _ = oracle.cgnr(u, src / scale, 0.11, dims, tol=1e-13)
+        assert oracle.rel_err(lat.unpack(x) / scale, want) < 1e-9

@@ -206,3 +206,55 @@ def test_fp64_arithmetic_has_its_own_launch_shape():
     assert lat.tiles(0, 1) == (64, 1, 1)
     lat.set_gauge(U, recon=12)
     assert lat.tiles(0, 1) == (64, 1, 1)
+
+
+def spread(psi, decades, seed):
+    """psi with its sites scaled by 10^(+-decades)."""
+    s = 10.0 ** (decades * (2.0 * gen.uniform(seed, gen.STREAM_MISC, 0, psi.shape[0]) - 1.0))
+    return psi * s[:, None, None]
+
+
+def test_rows_of_very_different_magnitude():
+    """Three right-hand sides, each in its own units: the bound of each site in its own row."""
+    U = gen.haar_links(DIMS, seed=3)
+    B = gen.gaussian_source(DIMS, seed=4, nrhs=3)
+    B = np.stack([spread(B[0], 20, 5), B[1] * 1e-200, spread(B[2], 3, 6) * 1e200])
+    lat = lattice(U)
+    fo = lat.new_field(nrhs=3)
+    lat.apply(KAPPA, lat.pack(B), fo, nrhs=3)
+    got = lat.unpack(fo, nrhs=3, squeeze=False)
+    for k in range(3):
+        err = np.abs(got[k] - oracle.apply_D(U, B[k], KAPPA, DIMS)).reshape(len(B[k]), -1).max(1)
+        assert np.all(err <= 2e-15 * neighbourhood_max(B[k], DIMS))
+
+
+@pytest.mark.parametrize("decades", [0, 3, 20])
+@pytest.mark.parametrize("bad_link", [False, True])
+def test_checkerboard_hops_of_different_magnitudes(decades, bad_link):
+    """The even-odd operator 1 - kappa^2 H_eo H_oe on sites of very different magnitude, unitary
+    links and not: D on the even field gives the odd half -kappa H_oe, D on that the even half; two
+    hops, each with the bound above (2e-15 of the largest value within two sites)."""
+    dims = (4, 4, 2, 6)
+    U = gen.haar_links(dims, seed=3)
+    if bad_link:
+        U[1, 9] *= 1.5
+    psi = spread(gen.gaussian_source(dims, seed=4), decades, 5)
+    x, y, z, t = np.meshgrid(*[np.arange(n) for n in dims], indexing="ij")
+    odd = ((x + y + z + t) & 1).transpose(3, 2, 1, 0).reshape(-1).astype(bool)
+    even_in = np.where(odd[:, None, None], 0.0, psi)
+    lat = lattice(U, dims)
+    for dagger in (False, True):
+        fo = lat.new_field()
+        lat.apply_schur(KAPPA, lat.pack(psi), fo, dagger=dagger)
+        got = lat.unpack(fo)
+        # D takes an even field to -kappa H_oe of it on the odd sites, and that to kappa^2 H_eo H_oe
+        h = oracle.apply_D(U, even_in, KAPPA, dims, dagger=dagger)
+        h[~odd] = 0
+        want = even_in - oracle.apply_D(U, h, KAPPA, dims, dagger=dagger)
+        near = neighbourhood_max(even_in, dims).reshape(*dims[::-1])
+        near2 = near.copy()
+        for ax in range(4):
+            near2 = np.maximum(near2, np.maximum(np.roll(near, 1, ax), np.roll(near, -1, ax)))
+        err = np.abs(got - want).reshape(len(psi), -1).max(1)
+        assert np.all(err[~odd] <= 4e-15 * near2.reshape(-1)[~odd])
+        assert np.all(got[odd] == 0)
