@@ -79,8 +79,9 @@ typedef enum wd_status {
  *            largest component of a site's neighbours: links are held to 2^-56, spinor
  *            components to 2^-62 and a site's hop sums to some 2^-54 of the unit, absolutely
  *            and not each relative to itself.  A site with a complex sum below 2^-14 of the
- *            unit, where a component below 2^-12 of it takes part, is computed with IEEE
- *            arithmetic (on the links as held); so are sites with spinors beyond
+ *            unit, to one of whose spins a colour below 2^-12 of it contributes, is computed
+ *            with IEEE arithmetic (on the links as held; not where all colours of that spin
+ *            are below 2^-45, which rounding leaves); so are sites with spinors beyond
  *            2^-894 .. 2^1007, other links and recon 8.  In norm, on random SU(3) links and
  *            Gaussian spinors, the operator's relative error is no larger than with IEEE
  *            arithmetic (6.2e-17 against 8.2e-17 at kappa = 0.12).

@@ -930,14 +930,15 @@ __device__ __noinline__ void half_native(const Geom &g, const void *in, const vo
     hopping_half<F64, RECON, DAG, EO, NC, true>(g, in, gauge, gdir_bytes, s, hh, acc);
 }
 
-// Whether the lane's eight hops read a complex component that is not zero but below
-// 2^-kFxSpreadBits of the unit of exponent E.  Out of line: rarely called.
+// How large the spinors are that the lane's hops read, colour by colour (fx_class; the larger of both
+// spins and of all hops), two bits each: over the hops of mu = 0, 1 at bit 2 b, of mu = 2, 3 at bit 6 + 2 b.
+// Out of line: rarely called.
 template <bool EO, bool NC>
-__device__ __noinline__ bool fx_spread(const Geom &g, const void *in, int s, int hh, int E) {
+__device__ __noinline__ unsigned fx_classes(const Geom &g, const void *in, int s, int hh, int E) {
     int xc[4], m = s;
     if constexpr (EO) m = eo_full_index(g, s, xc[0], xc[1], xc[2], xc[3]);
     else site_xyzt(g, s, xc[0], xc[1], xc[2], xc[3]);
-    bool found = false;
+    unsigned top[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int mu = k >> 1, L = g.L[mu], st = g.stride[mu], c = xc[mu];
@@ -951,10 +952,29 @@ __device__ __noinline__ bool fx_spread(const Geom &g, const void *in, int s, int
             C<double> p[3];
             load_spin<F64, NC>(in, g.Vs, n, h == 0 ? hh : mu < 2 ? 3 - hh : 2 + hh, p);
 #pragma unroll
-            for (int j = 0; j < 3; ++j) found |= fx_below(p[j].re, p[j].im, E);
+            for (int j = 0; j < 3; ++j) {
+                unsigned &t = top[3 * (mu >> 1) + j];
+                t = max(t, max((unsigned)__double2hiint(p[j].re) << 1, (unsigned)__double2hiint(p[j].im) << 1));
+            }
         }
     }
-    return found;
+    unsigned r = 0;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) r |= fx_class(top[j], E) << 2 * j;
+    return r;
+}
+// whether the hops of classes a and b (three colours each) feed a spin that has a colour far below the
+// unit without all of it being noise
+__device__ __forceinline__ bool fx_small_colour(unsigned a, unsigned b) {
+    unsigned most = 0;
+    bool small = false;
+#pragma unroll
+    for (int j = 0; j < 6; j += 2) {
+        const unsigned c = max(a >> j & 3u, b >> j & 3u);
+        most = max(most, c);
+        small |= c == 1u || c == 2u;
+    }
+    return small && most >= 2u;
 }
 
 // The hopping sum of site s for the spins this lane owns (hh and 3 - hh), zero where `on` is
@@ -984,7 +1004,7 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
             own[3 + k] = C<R>{fx_value(acc.v[6 + 2 * k], e), fx_value(acc.v[7 + 2 * k], e)};
         }
         // Sums far below the unit have few digits left.  That is no loss where large terms cancelled,
-        // but it is where the terms were small, and others, which do not enter this component (links
+        // but it is where all terms were small, and others, which do not enter this component (links
         // that do not mix colours, the other spin of a chirality), set the unit.
         unsigned low = ~0u;
 #pragma unroll
@@ -994,7 +1014,11 @@ __device__ __forceinline__ void hopping_own(const Geom &g, const void *in, const
         bool small = low < 2u * kFxSmallHi && acc.E >= kFxMinExp, native = acc.bad;
         if (__any_sync(0xffffffffu, small || native)) {
             small |= __shfl_xor_sync(0xffffffffu, small, 16) != 0;  // both lanes' spinors make both lanes' sums
-            if (on && small) native |= fx_spread<EO, NC>(g, in, s, hh, acc.E);
+            // the upper spin takes all of the lane's hops, the lower one its own of mu = 0, 1 and the partner's
+            // of mu = 2, 3
+            const unsigned cls = on && small ? fx_classes<EO, NC>(g, in, s, hh, acc.E) : 0u,
+                           partner = __shfl_xor_sync(0xffffffffu, cls, 16);
+            native |= fx_small_colour(cls, cls >> 6) || fx_small_colour(cls, partner >> 6);
             native |= __shfl_xor_sync(0xffffffffu, native, 16) != 0;
             if (__any_sync(0xffffffffu, native)) {
                 C<double> acc9[9];

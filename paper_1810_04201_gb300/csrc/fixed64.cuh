@@ -43,10 +43,12 @@ constexpr float kFxSmallToAcc = 0x1p-35f;        // small products come in units
 constexpr int kFxMinExp = 128, kFxMaxExp = 2030;
 
 // A site with a complex sum whose parts are both below 2^-kFxSmallBits units is redone in FP64 where
-// a complex component that entered its lanes' hops, zeros apart, is below 2^-kFxSpreadBits units
-// (hopping_own).  On Gaussian fields one warp in two million gets as far as looking at the inputs;
-// with the real and imaginary parts each by itself one in a hundred did, and 16^4 took 71 us for 32.
-constexpr int kFxSmallBits = 14, kFxSpreadBits = 12;
+// one colour of all spinors that a spin of its sums takes is below 2^-kFxSpreadBits units and not zero,
+// unless every colour is below 2^-kFxNoiseBits, as rounding leaves it where a projection cancels (around
+// a point source half of the sums are such: with them redone a 24^3 x 48 FP64 solve took 40.4 ms for 33.6).
+// On Gaussian fields one warp in two million gets as far as looking at the spinors; with the real and
+// imaginary parts of a sum each by itself one in a hundred did, and 16^4 took 71 us for 32.
+constexpr int kFxSmallBits = 14, kFxSpreadBits = 12, kFxNoiseBits = 45;
 constexpr int kFxSmallHi = 1 << (kFxAccBits - kFxSmallBits - 32);  // that sum's high word
 
 // a float of given bits and a float's bits, on either side (the arithmetic of a link is also compiled
@@ -116,11 +118,11 @@ __device__ __forceinline__ void fx_sum(double a, int ma, double b, int mb, unsig
              (long long)(fx_fixed(b, c) ^ (unsigned long long)(long long)mb) - (ma + mb), h, l);
 }
 
-// re + i im is not zero, but both parts are below 2^-kFxSpreadBits units of exponent E
-__device__ __forceinline__ bool fx_below(double re, double im, int E) {
-    const unsigned long long r = (unsigned long long)__double_as_longlong(re) << 1,
-                             i = (unsigned long long)__double_as_longlong(im) << 1, m = r > i ? r : i;
-    return m != 0 && (int)(m >> 53) <= E - kFxSpreadBits;
+// a magnitude, given as twice a high word, in units of exponent E: 0 zero (or below 2^-1042), 1 below
+// 2^-kFxNoiseBits, 2 below 2^-kFxSpreadBits, 3 larger
+__device__ __forceinline__ unsigned fx_class(unsigned hi2, int E) {
+    const int e = (int)(hi2 >> 21);
+    return hi2 == 0 ? 0u : e <= E - kFxNoiseBits ? 1u : e <= E - kFxSpreadBits ? 2u : 3u;
 }
 
 __host__ __device__ __forceinline__ long long fx_mac(int a, int b, long long s) { return (long long)a * b + s; }
