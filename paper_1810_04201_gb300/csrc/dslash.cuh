@@ -757,7 +757,8 @@ template <class R> __device__ __forceinline__ void exchange_halves(C<R> (&acc)[9
 // shifts the sums down.  The directions of a lower spin that goes to the partner lane come
 // first, so that a lane holds two spins of sums and not three.  FP64 arithmetic remains for half
 // of the projections, the final sums as doubles and for spinors that this cannot take (non-finite,
-// huge or tiny), whose sites go through half_native.  Recon-8 links and links that are not unitary
+// huge, tiny, or with a colour far below the others: kFxSmallBits), whose sites go through
+// half_native.  Recon-8 links and links that are not unitary
 // have kernels in FP64 arithmetic (dslash_kernel with FX = false).
 struct FxAcc {
     long long v[12];  // upper spin hh, then the lower spin under way: 3 x (re, im) each

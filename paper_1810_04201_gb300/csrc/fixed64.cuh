@@ -16,11 +16,11 @@
 // spinors: kappa 0.12 8.2e-17 -> 6.2e-17, kappa 1 1.57e-16 -> 1.01e-16, recon-12 at kappa 0.12
 // 1.06e-16 -> 9.1e-17).  A component far below the unit is not: what that could lose goes through
 // FP64 arithmetic (kFxSmallBits below).
-// Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 811-850 us (128- and 64-thread blocks),
-// 16^4 107 -> 34.5 us; with recon-12 links 5066 -> 1083 us.  (Three integer products of 29-bit
-// limbs per real product, the first form: 882-888, 36.5 and 1400 us.)  What bounds it now is the
-// latency of its integer and FP64 results with 16 warps per SM: on 32^3 x 64 the integer, multiply-
-// add and FP64 pipes are busy 47, 39 and 38 % of the cycles, DRAM 32 %, issue slots 50 %.
+// Measured, one Dslash with L2 flushed: 32^3 x 64 3090 -> 838 us (256-thread blocks; 64: 857),
+// 16^4 107 -> 37 us; with recon-12 links 5066 -> 978 us.  (Three integer products of 29-bit limbs per
+// real product, the first form: 882-888, 36.5 and 1400 us.)  What bounds it now is the latency of its
+// integer and FP64 results with 16 warps per SM: on 32^3 x 64 the integer, multiply-add and FP64 pipes
+// are busy 48, 40 and 39 % of the cycles, the XU pipe 2 %, DRAM 32 %, issue slots 51 %.
 //
 // Bounds.  A spinor component is a sum of two doubles, each below (1 - 2^-21) units, so H fits 32
 // bits; |L| <= 2^31 (a rebuilt row's 2^31 + 2^10); links |H| <= 2^30 (1 + 2^-11) with rows and columns of
