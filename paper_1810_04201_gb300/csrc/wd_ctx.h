@@ -19,7 +19,7 @@ struct wd_ctx {
     void *gauge_eo[wd::kNumPrec] = {};                 // checkerboard copies, per precision
     // whether a copy holds the current links, and the compression it has: new links or another
     // compression leave the buffers (solver graphs hold their addresses) until gauge_get fills or
-    // replaces them
+    // replaces them, or the context allocates something else and frees what is stale
     bool gauge_ok[wd::kNumPrec] = {}, gauge_eo_ok[wd::kNumPrec] = {};
     int gauge_recon[wd::kNumPrec] = {}, gauge_eo_recon[wd::kNumPrec] = {};
     double *gauge_canon = nullptr;                     // FP64 canonical copy on device
